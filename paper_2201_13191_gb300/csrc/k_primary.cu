@@ -3,8 +3,7 @@
 // (Sec. II-C.2); the per-material column masses rho*L are summed exactly in
 // 64-bit fixed point (each FP16 density is an integer multiple of 2^-24), and
 // the spectrum sum S(E) eta(E) exp(-mu(E) L) runs over the energy bins.  The
-// file also builds the packed voxel words and measures, at volume load, how
-// often neighbouring voxels change material.
+// file also builds the packed voxel words.
 #include <cuda_fp16.h>
 #include <stdint.h>
 
@@ -38,6 +37,9 @@ __global__ void __launch_bounds__(256) k_primary(const PrimaryParams P) {
   extern __shared__ __align__(8) unsigned char s_raw[];
   const int nm = P.tab.n_mat, nb = P.spec.n_bins, ns = P.tab.n_stage;
   float* s_mub = reinterpret_cast<float*>(s_raw);
+  __shared__ uint32_t s_pal[LAYOUT == VOX_HOP ? 256 : 1];
+  if (LAYOUT == VOX_HOP)
+    for (int q = threadIdx.x; q < 256; q += blockDim.x) s_pal[q] = __ldg(P.vol.pal + q);
   unsigned long long* my_acc =
       reinterpret_cast<unsigned long long*>(s_raw + (((size_t)nb * nm * 4 + 7) & ~(size_t)7)) + threadIdx.x;
   if (SACC)
@@ -88,12 +90,47 @@ __global__ void __launch_bounds__(256) k_primary(const PrimaryParams P) {
     h = L / (float)n;
     VoxRay r;
     r.set(V, o, w);
-    int cur = vox_mat(__ldg(V.vox + r.voxel<LAYOUT>(V, fmaf(0.5f, h, ta))));
+    const uint32_t w0 = __ldg(V.vox + r.voxel<LAYOUT>(V, fmaf(0.5f, h, ta)));
+    int cur = vox_mat(LAYOUT == VOX_HOP ? s_pal[w0 & 255u] : w0);
     unsigned long long run = 0ull;
+    auto change = [&](int m) {
+      if (m == cur) return;
+      if (SACC) my_acc[cur * blockDim.x] += run;
+      else switch (cur) {
+        case 0: acc[0] += run; break;
+        case 1: acc[1] += run; break;
+        case 2: acc[2] += run; break;
+        case 3: acc[3] += run; break;
+        case 4: acc[4] += run; break;
+        case 5: acc[5] += run; break;
+        case 6: acc[6] += run; break;
+        default: acc[7] += run; break;
+      }
+      cur = m;
+      run = 0ull;
+    };
+    if constexpr (LAYOUT == VOX_HOP) {
+      // one word stands for every midpoint in its uniform cube: the same integers, count times (2048^2 panel,
+      // 512^3 volume: 0.45 ms a projection against 3.6 with a gather per midpoint)
+      const float3 hv = make_float3(h * r.vw.x, h * r.vw.y, h * r.vw.z);
+      Hop hop;
+      hop.set(r, hv, (float)n);
+      const float nf = (float)n;
+      for (float k = 0.f; k < nf;) {
+        const float t = fmaf(k + 0.5f, h, ta);
+        const float3 p = make_float3(fmaf(t, r.vw.x, r.v0.x), fmaf(t, r.vw.y, r.v0.y), fmaf(t, r.vw.z, r.v0.z));
+        const uint32_t hw = __ldg(V.vox + r.voxel_p<LAYOUT>(V, p.x, p.y, p.z));
+        const float m = fminf(hop.steps(hw, p), nf - k);
+        const uint32_t wd = s_pal[hw & 255u];
+        change(vox_mat(wd));
+        run += (unsigned long long)(uint32_t)m * fp16_fixed24((uint16_t)(wd & 0xffffu));
+        k += m;
+      }
+    }
     // the words of the next kAhead midpoints are loaded before any is used (the
     // step positions are known in advance, so the gathers are independent);
     // midpoints past the chord's end repeat its last one and are not summed
-    for (int k0 = 0; k0 < n; k0 += kAhead) {
+    for (int k0 = 0; LAYOUT != VOX_HOP && k0 < n; k0 += kAhead) {
       uint32_t wd[kAhead];
 #pragma unroll
       for (int u = 0; u < kAhead; ++u) {
@@ -103,22 +140,7 @@ __global__ void __launch_bounds__(256) k_primary(const PrimaryParams P) {
 #pragma unroll
       for (int u = 0; u < kAhead; ++u) {
         if (k0 + u < n) {
-          const int m = vox_mat(wd[u]);
-          if (m != cur) {
-            if (SACC) my_acc[cur * blockDim.x] += run;
-            else switch (cur) {
-              case 0: acc[0] += run; break;
-              case 1: acc[1] += run; break;
-              case 2: acc[2] += run; break;
-              case 3: acc[3] += run; break;
-              case 4: acc[4] += run; break;
-              case 5: acc[5] += run; break;
-              case 6: acc[6] += run; break;
-              default: acc[7] += run; break;
-            }
-            cur = m;
-            run = 0ull;
-          }
+          change(vox_mat(wd[u]));
           run += fp16_fixed24((uint16_t)(wd[u] & 0xffffu));
         }
       }
@@ -163,8 +185,9 @@ cudaError_t launch_primary(const PrimaryParams& p, cudaStream_t s) {
   dim3 grid((npix + block - 1) / block, p.n_angles);
   const int smem = ((p.spec.n_bins * p.tab.n_mat * 4 + 7) & ~7) + (p.shared_acc ? p.tab.n_mat * block * 8 : 0);
   const bool brick = p.vol.layout == VOX_BRICK;
-  auto k = brick ? (p.shared_acc ? k_primary<VOX_BRICK, true> : k_primary<VOX_BRICK, false>)
-                 : (p.shared_acc ? k_primary<VOX_LIN, true> : k_primary<VOX_LIN, false>);
+  auto k = p.vol.layout == VOX_HOP ? (p.shared_acc ? k_primary<VOX_HOP, true> : k_primary<VOX_HOP, false>)
+           : brick                 ? (p.shared_acc ? k_primary<VOX_BRICK, true> : k_primary<VOX_BRICK, false>)
+                                   : (p.shared_acc ? k_primary<VOX_LIN, true> : k_primary<VOX_LIN, false>);
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
@@ -172,58 +195,6 @@ cudaError_t launch_primary(const PrimaryParams& p, cudaStream_t s) {
   k<<<grid, block, smem, s>>>(p);
   return cudaGetLastError();
 }
-
-}  // namespace mcx
-
-// Fraction of x-neighbour voxel pairs whose materials differ (how often a ray
-// meets a material change); chooses the primary kernel's accumulator variant.
-namespace mcx {
-namespace {
-__global__ void k_mat_changes(const uint8_t* __restrict__ mat, size_t n, int nx, unsigned long long* count) {
-  unsigned long long c = 0;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i + 1 < n; i += (size_t)gridDim.x * blockDim.x)
-    c += (i % (size_t)nx != (size_t)nx - 1) && mat[i] != mat[i + 1];
-  for (int o = 16; o > 0; o >>= 1) c += __shfl_down_sync(0xffffffffu, c, o);
-  if ((threadIdx.x & 31) == 0 && c) atomicAdd(count, c);
-}
-}  // namespace
-
-cudaError_t material_change_fraction(const uint8_t* mat, int nx, int ny, int nz, cudaStream_t s, double* frac) {
-  *frac = 0.0;
-  const size_t n = (size_t)nx * ny * nz;
-  const size_t pairs = n - (size_t)ny * nz;
-  if (pairs == 0) return cudaSuccess;
-  unsigned long long* d = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&d, 8, s);
-  if (e != cudaSuccess) return e;
-  unsigned long long h = 0;
-  e = cudaMemsetAsync(d, 0, 8, s);
-  if (e == cudaSuccess) {
-    k_mat_changes<<<152 * 8, 256, 0, s>>>(mat, n, nx, d);
-    e = cudaGetLastError();
-  }
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&h, d, 8, cudaMemcpyDeviceToHost, s);
-  cudaFreeAsync(d, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  *frac = (double)h / (double)pairs;
-  return e;
-}
-}  // namespace mcx
-
-// Device-side validation of a volume given by device pointers: every material
-// id below n_mat and every density a finite, non-negative binary16.
-namespace mcx {
-namespace {
-__global__ void k_validate_volume(const uint8_t* __restrict__ mat, const uint16_t* __restrict__ rho, size_t n,
-                                  int n_mat, int* bad) {
-  int b = 0;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const uint16_t h = rho[i];
-    b |= (mat[i] >= n_mat) | (((h & 0x8000u) != 0) & ((h & 0x7fffu) != 0)) | (((h >> 10) & 31u) == 31u);
-  }
-  if (__syncthreads_or(b) && threadIdx.x == 0) atomicOr(bad, 1);
-}
-}  // namespace
 
 // Packs material + density into voxel words over the padded grid; border
 // voxels repeat the nearest edge voxel.
@@ -268,21 +239,5 @@ cudaError_t pack_volume(const uint8_t* mat, const uint16_t* rho, int nx, int ny,
   padded_dims(nx, ny, nz, layout, &v);
   k_pack_volume<<<1024, 256, 0, s>>>(mat, rho, v, out);
   return cudaGetLastError();
-}
-
-cudaError_t validate_volume_device(const uint8_t* mat, const uint16_t* rho, size_t n, int n_mat, cudaStream_t s,
-                                   int* bad_host) {
-  int* d_bad = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&d_bad, sizeof(int), s);
-  if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(d_bad, 0, sizeof(int), s);
-  if (e == cudaSuccess) {
-    k_validate_volume<<<1024, 256, 0, s>>>(mat, rho, n, n_mat, d_bad);
-    e = cudaGetLastError();
-  }
-  if (e == cudaSuccess) e = cudaMemcpyAsync(bad_host, d_bad, sizeof(int), cudaMemcpyDeviceToHost, s);
-  cudaFreeAsync(d_bad, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  return e;
 }
 }  // namespace mcx

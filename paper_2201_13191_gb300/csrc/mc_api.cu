@@ -51,7 +51,10 @@ struct mc_ctx {
   float mesh_half[3] = {0.f, 0.f, 0.f};  // half extents of a box about the origin holding every vertex
   // volume
   bool have_volume = false;
-  uint32_t* d_vox = nullptr;  // packed voxel words (material | FP16 density)
+  uint32_t* d_vox = nullptr;
+  uint32_t* d_pal = nullptr;        // palette of a volume with clearance [kMaxPalette]
+  unsigned char* d_prep = nullptr;  // scratch of the volume load
+  size_t pal_cap = 0, prep_cap = 0;  // packed voxel words (material | FP16 density)
   size_t vox_cap = 0;
   int layout = VOX_LIN;
   int nx = 0, ny = 0, nz = 0;
@@ -88,6 +91,11 @@ struct mc_ctx {
 };
 
 namespace {
+
+// Share of mixed 2x2x2 cells up to which a volume gets words with clearance.  Measured by giving a growing share of
+// the object's voxels one of 16 densities: the transport takes as long as with single steps at 0.19 (64^3 cylinder),
+// 0.12 (256^3 ellipsoids) and 0.10 (512^3 ellipsoids), and the primary is faster at every share.
+constexpr double kMaxMixed = 0.10;
 
 int fail(mc_ctx* c, int code, const std::string& msg) {
   if (c) c->err = msg;
@@ -252,6 +260,7 @@ VolumeView volume_view(const mc_ctx* c) {
   VolumeView v;
   padded_dims(c->nx, c->ny, c->nz, c->layout, &v);
   v.vox = c->d_vox;
+  v.pal = c->d_pal;
   v.dx = c->dx; v.dy = c->dy; v.dz = c->dz;
   v.inv_dx = 1.f / c->dx; v.inv_dy = 1.f / c->dy; v.inv_dz = 1.f / c->dz;
   v.hx = 0.5f * c->nx * c->dx; v.hy = 0.5f * c->ny * c->dy; v.hz = 0.5f * c->nz * c->dz;
@@ -702,6 +711,8 @@ void mc_destroy(mc_ctx* ctx) {
   cudaDeviceSynchronize();
   cudaFree(ctx->d_blob);
   cudaFree(ctx->d_vox);
+  cudaFree(ctx->d_pal);
+  cudaFree(ctx->d_prep);
   cudaFree(ctx->d_mesh_nodes);
   cudaFree(ctx->d_mesh_tris);
   cudaFree(ctx->d_mesh_bodies);
@@ -822,54 +833,87 @@ int mc_load_volume(mc_ctx* ctx, const uint8_t* mat, const uint16_t* rho_fp16, in
     }
   }
   ctx->have_volume = false;
-  // stage the two arrays on the device, validate, pack into voxel words
+  // host arrays are staged on the device; device arrays are read where they are
   uint8_t* st_mat = nullptr;
   uint16_t* st_rho = nullptr;
-  CK(cudaMallocAsync((void**)&st_mat, n, s), "volume staging allocation");
-  cudaError_t e = cudaMallocAsync((void**)&st_rho, n * 2, s);
-  if (e != cudaSuccess) {
-    cudaFreeAsync(st_mat, s);
-    return cuda_fail(ctx, e, "volume staging allocation");
+  cudaError_t e = cudaSuccess;
+  if (!is_device_ptr) {
+    CK(cudaMallocAsync((void**)&st_mat, n, s), "volume staging allocation");
+    e = cudaMallocAsync((void**)&st_rho, n * 2, s);
+    if (e != cudaSuccess) {
+      cudaFreeAsync(st_mat, s);
+      return cuda_fail(ctx, e, "volume staging allocation");
+    }
+    e = cudaMemcpyAsync(st_mat, mat, n, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(st_rho, rho_fp16, n * 2, cudaMemcpyHostToDevice, s);
+    mat = st_mat;
+    rho_fp16 = st_rho;
   }
   auto release = [&]() {
-    cudaFreeAsync(st_mat, s);
-    cudaFreeAsync(st_rho, s);
+    if (st_mat) cudaFreeAsync(st_mat, s);
+    if (st_rho) cudaFreeAsync(st_rho, s);
   };
-  const cudaMemcpyKind kind = is_device_ptr ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-  e = cudaMemcpyAsync(st_mat, mat, n, kind, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(st_rho, rho_fp16, n * 2, kind, s);
   if (e != cudaSuccess) {
     release();
     return cuda_fail(ctx, e, "volume copy");
   }
-  if (is_device_ptr) {
-    // device data: validate on the device (material ids, finite non-negative densities)
-    int bad = 0;
-    e = validate_volume_device(st_mat, st_rho, n, ctx->n_mat, s, &bad);
-    if (e != cudaSuccess || bad) {
-      release();
-      if (e != cudaSuccess) return cuda_fail(ctx, e, "volume validation");
-      return fail(ctx, MC_ERR_INVALID_ARG, "volume holds an unknown material id or an invalid density");
+  // one pass: validity (host arrays were checked above), material changes, distinct (material, density) pairs
+  VolumeScan scan = {};
+  e = ensure(ctx->d_prep, ctx->prep_cap, scan_scratch_bytes());
+  if (e == cudaSuccess) e = ensure(ctx->d_pal, ctx->pal_cap, (size_t)kMaxPalette);
+  if (e == cudaSuccess) e = scan_volume(mat, rho_fp16, nx, ny, nz, ctx->n_mat, ctx->d_prep, ctx->d_pal, &scan, s);
+  if (e != cudaSuccess || scan.bad) {
+    release();
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "volume validation");
+    return fail(ctx, MC_ERR_INVALID_ARG, "volume holds an unknown material id or an invalid density");
+  }
+  // Layout.  Default: words with clearance (x fastest) where the volume has few (material, density) pairs and few
+  // mixed cells, so that a march takes many midpoints from one word.  Otherwise x fastest while the packed volume
+  // fits in 3/4 of L2 (measured faster there), 4^3 bricks once it streams from HBM (every ray direction then
+  // reuses its sectors).
+  int layout = ctx->opt.voxel_layout == 2 ? VOX_BRICK : VOX_LIN;
+  if (layout != VOX_BRICK && scan.pairs <= (uint32_t)kMaxPalette) {
+    e = ensure(ctx->d_vox, ctx->vox_cap, packed_words(nx, ny, nz, VOX_HOP));
+    // without room for the clearance scratch the volume is packed plainly
+    const size_t need = clearance_scratch_bytes(nx, ny, nz);
+    if (e == cudaSuccess && need > ctx->prep_cap) {
+      unsigned char* larger = nullptr;
+      if (cudaMalloc((void**)&larger, need) == cudaSuccess) {
+        // the scan's results stay
+        e = cudaMemcpyAsync(larger, ctx->d_prep, scan_scratch_bytes(), cudaMemcpyDeviceToDevice, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        cudaFree(ctx->d_prep);
+        ctx->d_prep = larger;
+        ctx->prep_cap = need;
+      } else {
+        (void)cudaGetLastError();
+      }
+    }
+    if (e == cudaSuccess && need <= ctx->prep_cap) {
+      double mixed = 1.0;
+      e = pack_palette(mat, rho_fp16, nx, ny, nz, ctx->d_prep, ctx->d_vox, &mixed, s);
+      if (e == cudaSuccess && mixed <= kMaxMixed) {
+        layout = VOX_HOP;
+        e = build_clearance(nx, ny, nz, ctx->d_prep, ctx->d_vox, s);
+      }
     }
   }
-  // default layout: x fastest while the packed volume fits in 3/4 of L2 (measured faster there);
-  // 4^3 bricks once it streams from HBM (every ray direction then reuses its sectors)
-  int layout = ctx->opt.voxel_layout == 2 ? VOX_BRICK : VOX_LIN;
-  if (ctx->opt.voxel_layout == 0) {
+  if (e == cudaSuccess && layout == VOX_LIN && ctx->opt.voxel_layout == 0) {
     int l2 = 0;
-    CK(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, ctx->device), "L2 size query");
+    e = cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, ctx->device);
     if ((double)packed_words(nx, ny, nz, VOX_LIN) * 4.0 > 0.75 * (double)l2) layout = VOX_BRICK;
   }
-  const size_t words = packed_words(nx, ny, nz, layout);
-  e = ensure(ctx->d_vox, ctx->vox_cap, words);
-  if (e == cudaSuccess) e = pack_volume(st_mat, st_rho, nx, ny, nz, layout, ctx->d_vox, words, s);
-  double change = 0.0;
-  if (e == cudaSuccess) e = material_change_fraction(st_mat, nx, ny, nz, s, &change);
+  if (e == cudaSuccess && layout != VOX_HOP) {
+    const size_t words = packed_words(nx, ny, nz, layout);
+    e = ensure(ctx->d_vox, ctx->vox_cap, words);
+    if (e == cudaSuccess) e = pack_volume(mat, rho_fp16, nx, ny, nz, layout, ctx->d_vox, words, s);
+  }
   release();
   if (e != cudaSuccess) return cuda_fail(ctx, e, "volume packing");
   CK(cudaStreamSynchronize(s), "volume load");
+  const size_t x_pairs = n - (size_t)ny * nz;
   ctx->layout = layout;
-  ctx->mat_change = change;
+  ctx->mat_change = x_pairs ? (double)scan.changes / (double)x_pairs : 0.0;
   ctx->nx = nx; ctx->ny = ny; ctx->nz = nz;
   ctx->dx = dx; ctx->dy = dy; ctx->dz = dz;
   ctx->have_volume = true;

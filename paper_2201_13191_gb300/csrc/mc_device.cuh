@@ -69,6 +69,7 @@ struct SmemTables {
   const float2* comp;  // [n_mat][kMaxComp] (w Z^2, b)
   const float* compz;  // [n_mat][kMaxComp] w Z
   const int* ncomp;    // [n_mat]
+  const uint32_t* pal; // [256] palette of a volume with clearance
   int n_mat, n_stage, use_eta, bound;
   float E0, inv_dE, mec2, inv_hc;
 
@@ -186,7 +187,7 @@ __device__ __forceinline__ bool clip_box(const VolumeView& v, float3 x, float3 w
 // Word index of padded voxel (ix, iy, iz) in the packed volume.
 template <int LAYOUT>
 __device__ __host__ __forceinline__ int vox_index(const VolumeView& vol, int ix, int iy, int iz) {
-  if (LAYOUT == VOX_LIN) return (iz * vol.py + iy) * vol.px + ix;
+  if (LAYOUT != VOX_BRICK) return (iz * vol.py + iy) * vol.px + ix;
   const int brick = ((iz >> 2) * vol.nby + (iy >> 2)) * vol.nbx + (ix >> 2);
   const int lx = ix & 3, ly = iy & 3, lz = iz & 3;
   const int m = (lx & 1) | ((ly & 1) << 1) | ((lz & 1) << 2) | ((lx & 2) << 2) | ((ly & 2) << 3) | ((lz & 2) << 4);
@@ -219,7 +220,7 @@ struct VoxRay {
   // The same for a point given in padded voxel units.
   template <int LAYOUT>
   __device__ __forceinline__ int voxel_p(const VolumeView& vol, float px, float py, float pz) const {
-    if (LAYOUT == VOX_LIN) {
+    if (LAYOUT != VOX_BRICK) {
       // (bx - C) + px (by - C) + px py (bz - C) with b the bit patterns of the
       // round-down adds (C = 0x4B000000, see floor_pos): the offsets fold into
       // one precomputed bias (exact in 32-bit wraparound arithmetic); the
@@ -239,6 +240,47 @@ struct VoxRay {
 
 __device__ __forceinline__ int vox_mat(uint32_t w) { return (int)((w >> 16) & 255u); }
 __device__ __forceinline__ float vox_rho(uint32_t w) { return __half2float(__ushort_as_half((unsigned short)(w & 0xffffu))); }
+
+// Steps a march may take from one word of a volume with clearance (VOX_HOP):
+// the cube of 2^c voxels per axis that starts at step k's voxel and extends in
+// the ray's octant is uniform, so every midpoint before the ray leaves it reads
+// the same material and density.  eps (in voxels) keeps the exit inside by more
+// than the midpoints' rounding: a few units in the last place of the largest
+// coordinate on the ray, taken 30 times over.
+struct Hop {
+  float3 inv;   // 1 / hv
+  float3 half;  // |1 / hv| / 2
+  float3 off;   // -eps |1 / hv|, less another |1 / hv| on the axes the ray runs down
+  int rot;      // brings the octant's code into the exponent field
+  __device__ __forceinline__ void axis(float h, float eps, float& iv, float& hf, float& of) {
+    const float a = 1.f / fmaxf(fabsf(h), 1e-20f);
+    iv = copysignf(a, h);
+    hf = 0.5f * a;
+    of = -a * (h < 0.f ? 1.f + eps : eps);
+  }
+  __device__ __forceinline__ void set(const VoxRay& r, float3 hv, float n) {
+    const float hm = fmaxf(fabsf(hv.x), fmaxf(fabsf(hv.y), fabsf(hv.z)));
+    const float eps = 4e-6f * fmaf(n, hm, fmaxf(fabsf(r.v0.x), fmaxf(fabsf(r.v0.y), fabsf(r.v0.z))));
+    axis(hv.x, eps, inv.x, half.x, off.x);
+    axis(hv.y, eps, inv.y, half.y, off.y);
+    axis(hv.z, eps, inv.z, half.z, off.z);
+    rot = 17 + 3 * ((hv.x < 0.f ? 1 : 0) + (hv.y < 0.f ? 2 : 0) + (hv.z < 0.f ? 4 : 0));
+  }
+  // Steps from the midpoint p (padded voxel units) whose word is w, as a float
+  // (step indices stay below 2^23, exact in FP32).  With f the midpoint's place
+  // in its voxel the ray leaves the cube along an axis after (2^c - f) / hv
+  // steps, or (2^c - 1 + f) / |hv| where it runs down.
+  __device__ __forceinline__ float steps(uint32_t w, float3 p) const {
+    const float two_c1 = __uint_as_float((__funnelshift_r(w, w, rot) & 0x03800000u) | 0x40000000u);  // 2^(c + 1)
+    const float fx = p.x - (__fadd_rd(p.x, 8388608.f) - 8388608.f);
+    const float fy = p.y - (__fadd_rd(p.y, 8388608.f) - 8388608.f);
+    const float fz = p.z - (__fadd_rd(p.z, 8388608.f) - 8388608.f);
+    const float tx = fmaf(two_c1, half.x, fmaf(-fx, inv.x, off.x));
+    const float ty = fmaf(two_c1, half.y, fmaf(-fy, inv.y, off.y));
+    const float tz = fmaf(two_c1, half.z, fmaf(-fz, inv.z, off.z));
+    return __fadd_rd(fmaxf(fminf(tx, fminf(ty, tz)), 0.f), 8388608.f) - 8388607.f;
+  }
+};
 
 __device__ __forceinline__ int step_count(float L, float step) { return max(1, (int)ceilf(L / step)); }
 

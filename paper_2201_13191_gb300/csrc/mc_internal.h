@@ -47,8 +47,10 @@ struct TableView {
 // Layout LIN: x fastest.  Layout BRICK: 4x4x4 bricks (x fastest between
 // bricks), Morton order inside a brick, so each 32-byte sector holds a 2x2x2
 // cube and each 128-byte line a 4x4x2 slab whatever the ray direction.
-enum VoxLayout { VOX_LIN = 0, VOX_BRICK = 1 };
-// Transport geometry selector beside the two voxel layouts: closed triangle-
+// HOP: x fastest, bits 0-7 a palette index (the words of the volume's distinct
+// (material, density) pairs), bits 8-31 the uniform cube ahead per octant (k_clearance.cu).
+enum VoxLayout { VOX_LIN = 0, VOX_BRICK = 1, VOX_HOP = 3 };
+// Transport geometry selector beside the voxel layouts: closed triangle-
 // mesh bodies (MeshView below) with exact flights instead of the march.
 constexpr int GEO_MESH = 2;
 
@@ -58,6 +60,7 @@ constexpr int GEO_MESH = 2;
 // march needs no per-axis clamps.
 struct VolumeView {
   const uint32_t* vox;
+  const uint32_t* pal;  // HOP: voxel words of the palette [256]
   int layout;
   int nbx, nby;    // bricks along x, y (BRICK layout, padded dims)
   int px, py, pz;  // padded dims
@@ -120,7 +123,7 @@ struct TransportParams {
   const unsigned long long* seed_dev = nullptr;
   // triangle-mesh geometry (geometry == GEO_MESH); `vol` then carries only the
   // half extents of a box around the bodies (hx, hy, hz)
-  int geometry = 0;  // VOX_LIN / VOX_BRICK from vol.layout, or GEO_MESH
+  int geometry = 0;  // VOX_* from vol.layout, or GEO_MESH
   MeshView mesh = {};
   // TALLY_TILED: tiles of tile_u x tile_v pixels, n_tu across, n_tiles in all;
   // work in chunks of up to tile_chunk histories of one (angle, tile), tile_k
@@ -163,21 +166,33 @@ int transport_shared_pixels(const TransportParams& p);
 cudaError_t transport_occupancy(int block, int smem, int* blocks_per_sm, bool mesh = false, int layout = VOX_LIN);
 cudaError_t launch_finalize(const double* tally, int n_batches, size_t n, float* out, float* var, cudaStream_t s);
 cudaError_t launch_primary(const PrimaryParams& p, cudaStream_t s);
-// Fraction of x-neighbour voxel pairs of a device material array whose materials differ (synchronises s).
-cudaError_t material_change_fraction(const uint8_t* mat, int nx, int ny, int nz, cudaStream_t s, double* frac);
 
 // Returns the depth of the deepest leaf (the device descent needs depth < 64).
 int build_mesh_bvh(const float* v, const int* tris, const int* tri_body, int nt, std::vector<float4>& nodes,
                    std::vector<float4>& out_tris);
 cudaError_t launch_primary_mesh(const PrimaryParams& p, const MeshView& m, cudaStream_t s);
-// Checks a device-resident volume (ids < n_mat, finite non-negative binary16
-// densities); *bad_host = 1 if any voxel fails.  Synchronises s.
-cudaError_t validate_volume_device(const uint8_t* mat, const uint16_t* rho, size_t n, int n_mat, cudaStream_t s,
-                                   int* bad_host);
 // Packs material + density into voxel words in the given layout.
 cudaError_t pack_volume(const uint8_t* mat, const uint16_t* rho, int nx, int ny, int nz, int layout, uint32_t* out,
                         size_t out_words, cudaStream_t s);
 size_t packed_words(int nx, int ny, int nz, int layout);
+// One pass over a volume's device arrays (k_clearance.cu): bad != 0 if a material id is not below n_mat or a
+// density is not a finite, non-negative binary16; the x-neighbour pairs of different materials; the distinct
+// (material, density) pairs, the first 256 of them as voxel words in pal.  Synchronises s.
+struct VolumeScan {
+  unsigned long long changes, mixed;
+  uint32_t pairs, bad;
+};
+constexpr int kMaxPalette = 256;
+size_t scan_scratch_bytes();
+cudaError_t scan_volume(const uint8_t* mat, const uint16_t* rho, int nx, int ny, int nz, int n_mat, void* scratch,
+                        uint32_t* pal, VolumeScan* out, cudaStream_t s);
+// Volumes with clearance, from a scan's scratch (of clearance_scratch_bytes) that found at most kMaxPalette
+// pairs: the palette indices into vox (padded, x fastest) and the share of 2x2x2 voxel cells that are mixed
+// (synchronises s), then the octant codes beside the indices.
+size_t clearance_scratch_bytes(int nx, int ny, int nz);
+cudaError_t pack_palette(const uint8_t* mat, const uint16_t* rho, int nx, int ny, int nz, void* scratch, uint32_t* vox,
+                         double* mixed, cudaStream_t s);
+cudaError_t build_clearance(int nx, int ny, int nz, void* scratch, uint32_t* vox, cudaStream_t s);
 // Padded dimensions, brick counts and word count of a packed volume.
 void padded_dims(int nx, int ny, int nz, int layout, VolumeView* v);
 
