@@ -20,7 +20,7 @@ OUT = os.path.join(HERE, "libmc.so")
 PROBE_OUT = os.path.join(HERE, "libmcprobe.so")
 BUILD = os.path.join(HERE, "_build")
 SOURCES = ["mc_api.cu", "k_transport.cu", "k_primary.cu", "k_post.cu", "k_static.cu", "k_conv.cu", "k_nn.cu",
-           "denoiser.cu", "k_recon.cu", "k_mesh.cu", "k_clearance.cu"]
+           "denoiser.cu", "k_recon.cu", "k_mesh.cu", "k_clearance.cu", "k_ramp.cu"]
 PROBE_SOURCES = ["probe/k_probe.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC"]

@@ -102,60 +102,131 @@ __global__ void __launch_bounds__(kFiltThreads) k_fdk_filter(const float* __rest
   }
 }
 
+// a / b, correctly rounded, from r = 1 / b (correctly rounded): the quotient a r
+// corrected by its remainder (Markstein, IBM J. Res. Dev. 34, 1990).
+__device__ __forceinline__ float div_by(float a, float b, float r) {
+  const float q = a * r;
+  return fmaf(fmaf(-q, b, a), r, q);
+}
+
 // Voxel-driven backprojection: f(x) = (dbeta / 2) sum_beta (D / (D - x.n))^2 q(u(x), v(x)),
-// q bilinearly interpolated at the voxel's projection (zero outside the panel).
-// Voxel-driven backprojection: each thread owns kZB voxels of one (x, y)
-// column; per projection the source-side terms (depth, magnification, u and
-// its bilinear weights) are computed once for the column, then each voxel adds
-// its bilinear sample (the same expressions as one voxel at a time, so the
-// same sums).
-constexpr int kZB = 4;
-__global__ void k_fdk_backproject(const float* __restrict__ q, const float* __restrict__ cb, const float* __restrict__ sb,
-                                  int n_proj, int nu, int nv, float du_iso, float dv_iso, float sod, int nx, int ny,
-                                  int nz, float dx, float dy, float dz, float scale, float* __restrict__ vol) {
-  const int nzb = (nz + kZB - 1) / kZB;
-  const size_t n = (size_t)nx * ny * nzb;
-  for (size_t i = gtid(); i < n; i += gstride()) {
-    const int ix = (int)(i % nx);
-    const size_t t = i / nx;
-    const int iy = (int)(t % ny), iz0 = (int)(t / ny) * kZB;
-    const float x = ((float)ix - 0.5f * (float)(nx - 1)) * dx;
-    const float y = ((float)iy - 0.5f * (float)(ny - 1)) * dy;
-    float z[kZB], acc[kZB];
+// q bilinearly interpolated at the voxel's projection (zero outside the panel);
+// the projections come in chunks, whose sums continue in vol (`first` starts
+// them, `scale` is 1 until the last).  Each thread owns ZB voxels of one (x, y) column; per projection the
+// source-side terms (depth, magnification, u and its bilinear weights) are
+// computed once for the column, then each voxel adds its bilinear sample (the
+// same expressions as one voxel at a time, so the same sums).  Bound by the L1
+// wavefronts of the four taps (3.5 per load): a warp owns 8 x 4 columns, whose
+// taps lie close together on the panel whatever the angle (a row of 32 in x
+// spreads over up to 130 panel pixels).  256^3 x 360 projections of 1024^2: 15.3
+// -> 9.3 ms with these tiles, the divisions by a stored reciprocal and ZB = 8.
+template <int ZB>
+__global__ void __launch_bounds__(256) k_fdk_backproject(const float* __restrict__ q, const float* __restrict__ cb,
+                                                         const float* __restrict__ sb, int n_proj, int nu, int nv,
+                                                         float du_iso, float dv_iso, float inv_du, float inv_dv,
+                                                         float sod, int nx, int ny, int nz, float dx, float dy, float dz,
+                                                         int first, float scale, float* __restrict__ vol) {
+  // blocks of 16 x 16 columns (2 x 4 warps), x fastest, then y, then z
+  const int bx_n = (nx + 15) / 16, by_n = (ny + 15) / 16;
+  const int bx = (int)(blockIdx.x % (unsigned)bx_n);
+  const unsigned byz = blockIdx.x / (unsigned)bx_n;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int ix = bx * 16 + (warp & 1) * 8 + (lane & 7);
+  const int iy = (int)(byz % (unsigned)by_n) * 16 + (warp >> 1) * 4 + (lane >> 3);
+  const int iz0 = (int)(byz / (unsigned)by_n) * ZB;
+  if (ix >= nx || iy >= ny) return;
+  const float x = ((float)ix - 0.5f * (float)(nx - 1)) * dx;
+  const float y = ((float)iy - 0.5f * (float)(ny - 1)) * dy;
+  const float cu = 0.5f * (float)(nu - 1), cv = 0.5f * (float)(nv - 1);
+  const float u_top = (float)(nu - 1), v_top = (float)(nv - 1);
+  constexpr float kFloor = 12582912.f;  // 1.5 x 2^23: a round-down add leaves floor in the low bits
+  float z[ZB], acc[ZB];
 #pragma unroll
-    for (int j = 0; j < kZB; ++j) {
-      z[j] = ((float)(iz0 + j) - 0.5f * (float)(nz - 1)) * dz;
-      acc[j] = 0.f;
-    }
-    for (int k = 0; k < n_proj; ++k) {
-      const float c = __ldg(cb + k), s = __ldg(sb + k);
-      const float depth = sod - (x * c + y * s);  // distance from the source along the central ray
-      const float mag = sod / depth;
-      const float u = (-x * s + y * c) * mag;     // isocentre-plane coordinates
-      const float fu = u / du_iso + 0.5f * (float)(nu - 1);
-      const int u0 = __float2int_rd(fu);
-      const float au = fu - (float)u0;
-      const bool u_in = u0 >= 0 && u0 + 1 < nu;
-      const float* qp = q + (size_t)k * nu * nv;
+  for (int j = 0; j < ZB; ++j) {
+    z[j] = ((float)(iz0 + j) - 0.5f * (float)(nz - 1)) * dz;
+    acc[j] = first || iz0 + j >= nz ? 0.f : vol[((size_t)(iz0 + j) * ny + iy) * nx + ix];
+  }
+  const size_t img = (size_t)nu * nv;
+#pragma unroll 1
+  for (int k = 0; k < n_proj; ++k, q += img) {
+    const float c = __ldg(cb + k), s = __ldg(sb + k);
+    const float depth = sod - (x * c + y * s);  // distance from the source along the central ray
+    const float mag = sod / depth;
+    const float u = (-x * s + y * c) * mag;     // isocentre-plane coordinates
+    const float fu = div_by(u, du_iso, inv_du) + cu;
+    // floor(fu) >= 0 and floor(fu) + 1 < nu (false for a NaN)
+    const bool u_in = fu >= 0.f && fu < u_top;
+    const float fl = __fadd_rd(fu, kFloor);
+    const int u0 = u_in ? __float_as_int(fl) - 0x4B400000 : 0;
+    const float au = fu - (fl - kFloor);
+    const float bu = 1.f - au, m2 = mag * mag;
+    if constexpr (ZB <= 2) {
+      // few warps: every tap is loaded before any is used (a voxel outside the panel reads a word it leaves out)
+      float av[ZB], t[ZB][4];
+      bool in[ZB];
 #pragma unroll
-      for (int j = 0; j < kZB; ++j) {
+      for (int j = 0; j < ZB; ++j) {
         const float v = z[j] * mag;
-        const float fv = v / dv_iso + 0.5f * (float)(nv - 1);
-        const int v0 = __float2int_rd(fv);
-        const float av = fv - (float)v0;
+        const float fv = div_by(v, dv_iso, inv_dv) + cv;
+        const float fw = __fadd_rd(fv, kFloor);
+        av[j] = fv - (fw - kFloor);
+        in[j] = u_in && fv >= 0.f && fv < v_top;
+        const float* r0 = q + (in[j] ? (__float_as_int(fw) - 0x4B400000) * nu + u0 : 0);
+        t[j][0] = __ldg(r0);
+        t[j][1] = __ldg(r0 + 1);
+        t[j][2] = __ldg(r0 + nu);
+        t[j][3] = __ldg(r0 + nu + 1);
+      }
+#pragma unroll
+      for (int j = 0; j < ZB; ++j) {
+        const float val = (1.f - av[j]) * (bu * t[j][0] + au * t[j][1]) + av[j] * (bu * t[j][2] + au * t[j][3]);
+        acc[j] = fmaf(m2, in[j] ? val : 0.f, acc[j]);
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < ZB; ++j) {
+        const float v = z[j] * mag;
+        const float fv = div_by(v, dv_iso, inv_dv) + cv;
+        const float fw = __fadd_rd(fv, kFloor);
+        const float av = fv - (fw - kFloor);
         float val = 0.f;
-        if (u_in && v0 >= 0 && v0 + 1 < nv) {
-          const float* r0 = qp + (size_t)v0 * nu + u0;
-          val = (1.f - av) * ((1.f - au) * __ldg(r0) + au * __ldg(r0 + 1)) +
-                av * ((1.f - au) * __ldg(r0 + nu) + au * __ldg(r0 + nu + 1));
+        if (u_in && fv >= 0.f && fv < v_top) {
+          const float* r0 = q + ((__float_as_int(fw) - 0x4B400000) * nu + u0);
+          const float* r1 = r0 + nu;
+          val = (1.f - av) * (bu * __ldg(r0) + au * __ldg(r0 + 1)) + av * (bu * __ldg(r1) + au * __ldg(r1 + 1));
         }
-        acc[j] = fmaf(mag * mag, val, acc[j]);
+        acc[j] = fmaf(m2, val, acc[j]);
       }
     }
-#pragma unroll
-    for (int j = 0; j < kZB; ++j)
-      if (iz0 + j < nz) vol[((size_t)(iz0 + j) * ny + iy) * nx + ix] = acc[j] * scale;
   }
+#pragma unroll
+  for (int j = 0; j < ZB; ++j)
+    if (iz0 + j < nz) vol[((size_t)(iz0 + j) * ny + iy) * nx + ix] = acc[j] * scale;
+}
+
+template <int ZB>
+cudaError_t backproject(const float* q, const float* cb, const float* sb, int n_proj, int nu, int nv, float du, float dv,
+                        float sod, int nx, int ny, int nz, float dx, float dy, float dz, bool first,
+                        float scale, float* vol, cudaStream_t s) {
+  const long long blocks = (long long)((nx + 15) / 16) * ((ny + 15) / 16) * ((nz + ZB - 1) / ZB);
+  if (blocks > 0x7FFFFFFFll) return cudaErrorInvalidValue;
+  k_fdk_backproject<ZB><<<(unsigned)blocks, 256, 0, s>>>(q, cb, sb, n_proj, nu, nv, du, dv, 1.f / du, 1.f / dv, sod, nx, ny,
+                                                         nz, dx, dy, dz, first ? 1 : 0, scale, vol);
+  return cudaGetLastError();
+}
+
+// Rows longer than the transforms of k_ramp.cu take.
+cudaError_t filter_direct(const float* p, int nu, int nv, int rows_total, float du, float dv, float sod, float* q,
+                          cudaStream_t s) {
+  const int span = kFiltThreads * kFiltOut;
+  const size_t npad = ((size_t)nu + span - 1) / span * span;
+  const size_t smem = ((2 * (npad + kFiltOut) + 1) + (size_t)kFiltRows * nu) * 4;
+  if (smem > 200 * 1024) return cudaErrorInvalidValue;
+  cudaError_t e = cudaFuncSetAttribute(k_fdk_filter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  k_fdk_filter<<<(rows_total + kFiltRows - 1) / kFiltRows, kFiltThreads, smem, s>>>(p, nu, nv, rows_total, du, dv, sod,
+                                                                                    q);
+  return cudaGetLastError();
 }
 
 // Histogram of vol over [lo, hi) in nbins bins (values outside are clamped to the end bins).
@@ -299,26 +370,26 @@ cudaError_t recon_log_norm(const float* I, const float* I0, size_t img, size_t n
 }
 
 cudaError_t recon_fdk(const float* p, int n_proj, const float* d_cos, const float* d_sin, int nu, int nv, float pu,
-                      float pv, float sod, float sdd, int nx, int ny, int nz, float dx, float dy, float dz, float* q_tmp,
-                      float* vol, cudaStream_t s) {
+                      float pv, float sod, float sdd, int nx, int ny, int nz, float dx, float dy, float dz,
+                      float* d_ramp, int chunk, float* q_tmp, float* vol, cudaStream_t s) {
   const float du = pu * sod / sdd, dv = pv * sod / sdd;  // pixel pitch at the isocentre
-  const int span = kFiltThreads * kFiltOut;
-  const size_t npad = ((size_t)nu + span - 1) / span * span;
-  const size_t smem = ((2 * (npad + kFiltOut) + 1) + (size_t)kFiltRows * nu) * 4;
-  if (smem > 200 * 1024) return cudaErrorInvalidValue;
-  cudaError_t e = cudaFuncSetAttribute(k_fdk_filter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  const int rows_total = n_proj * nv;
-  k_fdk_filter<<<(rows_total + kFiltRows - 1) / kFiltRows, kFiltThreads, smem, s>>>(p, nu, nv, rows_total, du, dv, sod,
-                                                                                    q_tmp);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
   // full orbit: (dbeta / 2) with dbeta = 2 pi / n_proj
   const float scale = 3.14159265358979f / (float)n_proj;
-  const size_t n = (size_t)nx * ny * ((nz + kZB - 1) / kZB);
-  k_fdk_backproject<<<blocks_for(n), 256, 0, s>>>(q_tmp, d_cos, d_sin, n_proj, nu, nv, du, dv, sod, nx, ny, nz, dx,
-                                                  dy, dz, scale, vol);
-  return cudaGetLastError();
+  const size_t img = (size_t)nu * nv;
+  // 8 voxels of a column per thread share its source-side terms; with fewer than about 16 blocks per SM of them, 2
+  // (200^3 x 128 projections, 4225 blocks: 1.56 / 1.72 ms with 8 / 2; 128^3 x 360, 1024 blocks: 2.2 / 1.7)
+  const bool deep = (long long)((nx + 15) / 16) * ((ny + 15) / 16) * ((nz + 7) / 8) >= 16ll * 152;
+  for (int k = 0; k < n_proj; k += chunk) {
+    const int m = n_proj - k < chunk ? n_proj - k : chunk;
+    cudaError_t e = d_ramp ? ramp_filter(p + k * img, nu, nv, m * nv, du, dv, sod, d_ramp, q_tmp, k == 0, s)
+                           : filter_direct(p + k * img, nu, nv, m * nv, du, dv, sod, q_tmp, s);
+    if (e != cudaSuccess) return e;
+    const float sc = k + m == n_proj ? scale : 1.f;
+    e = deep ? backproject<8>(q_tmp, d_cos + k, d_sin + k, m, nu, nv, du, dv, sod, nx, ny, nz, dx, dy, dz, k == 0, sc, vol, s)
+             : backproject<2>(q_tmp, d_cos + k, d_sin + k, m, nu, nv, du, dv, sod, nx, ny, nz, dx, dy, dz, k == 0, sc, vol, s);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t recon_otsu_segment(const float* vol, size_t n, float lo, float hi, int classes, const int* d_cls_mat,

@@ -228,9 +228,17 @@ cudaError_t launch_conv3x3_wgrad(const WgradParams& p, int splits, cudaStream_t 
 
 // Correction plumbing (k_recon.cu)
 cudaError_t recon_log_norm(const float* I, const float* I0, size_t img, size_t n, float* a, cudaStream_t s);
+// Ramp filter by transforms (k_ramp.cu): ramp_points: transform length for rows of nu values (0: rows longer than
+// 4096, filtered by direct sums); ramp_kernel: the summed kernel (host, ramp_points values); ramp: device, the summed
+// kernel followed by 4 ramp_points floats, the tables, which are made when `tables` is set.
+int ramp_points(int nu);
+void ramp_kernel(int nu, float du, float* g);
+cudaError_t ramp_filter(const float* p, int nu, int nv, int rows, float du, float dv, float sod, float* ramp, float* q,
+                        bool tables, cudaStream_t s);
+// d_ramp: as above (null when ramp_points(nu) == 0); q_tmp holds `chunk` filtered projections
 cudaError_t recon_fdk(const float* p, int n_proj, const float* d_cos, const float* d_sin, int nu, int nv, float pu,
-                      float pv, float sod, float sdd, int nx, int ny, int nz, float dx, float dy, float dz, float* q_tmp,
-                      float* vol, cudaStream_t s);
+                      float pv, float sod, float sdd, int nx, int ny, int nz, float dx, float dy, float dz,
+                      float* d_ramp, int chunk, float* q_tmp, float* vol, cudaStream_t s);
 cudaError_t recon_otsu_segment(const float* vol, size_t n, float lo, float hi, int classes, const int* d_cls_mat,
                                const float* d_cls_murho, const float* d_cls_rho0, float rho_max, unsigned int* d_hist,
                                int* d_thr, uint8_t* mat, uint16_t* rho, cudaStream_t s);
