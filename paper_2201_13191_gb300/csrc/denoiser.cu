@@ -33,9 +33,8 @@ namespace {
 struct Layer {
   int cin = 0, cout = 0;
   bool relu = true;
-  float *w = nullptr, *b = nullptr;    // FP32 master [cout][9][cin], [cout]
-  float *gw = nullptr, *gb = nullptr;  // gradients
-  float *mw = nullptr, *vw = nullptr, *mb = nullptr, *vb = nullptr;  // Adam moments
+  float *w = nullptr, *b = nullptr;    // FP32 master [cout][9][cin], [cout] (in Denoiser::par)
+  float *gw = nullptr, *gb = nullptr;  // gradients (in Denoiser::grad)
   __nv_bfloat16* wb = nullptr;  // forward weights, tensor-core order [cin/8][9][cout][8]
   __nv_bfloat16* wt = nullptr;  // adjoint weights, tensor-core order [cout/8][9][cin][8]
   size_t nw() const { return (size_t)cout * 9 * cin; }
@@ -58,8 +57,11 @@ struct Denoiser {
       *u1b, *cat0, *u0a, *u0b, *gbuf;
   float* out;  // FP32 [B][H][W][16]
   // gradients, FP32
-  float *g_out, *g_u0b, *g_u0a, *g_cat0up, *g_s0, *g_u1b, *g_u1a, *g_cat1up, *g_s1, *g_u2b, *g_u2a, *g_cat2up, *g_s2,
-      *g_a3b, *g_a3a, *g_p2, *g_a2a, *g_p1, *g_a1a, *g_p0, *g_a0a;
+  float *g_u0b, *g_u0a, *g_cat0up, *g_s0, *g_u1a, *g_cat1up, *g_s1, *g_u2a, *g_cat2up, *g_s2, *g_a3a, *g_p2, *g_a2a,
+      *g_p1, *g_a1a, *g_p0, *g_a0a;
+  // every layer's parameters (weights, then biases), gradients and Adam moments, each one array
+  float *par, *grad, *mom, *var;
+  nn::LayerTable table;
   float* scale;  // [B]
   double* loss;  // [1]
   int* err;      // [1]
@@ -134,34 +136,29 @@ cudaError_t forward(Denoiser* d, const float* img, int n, cudaStream_t s) {
   TRY(nn::pool_fwd(d->s2, n, d->H >> 2, d->W >> 2, 128, d->p2, s));
   TRY(c(6, d->p2, d->a3a));
   TRY(c(7, d->a3a, d->a3b));
-  TRY(nn::up_fwd(d->a3b, n, d->H >> 3, d->W >> 3, 256, d->cat2, 384, 0, s));
-  TRY(nn::copy_channels(d->s2, npix(d, n, 2), 128, d->cat2, 384, 256, s));
+  TRY(nn::up_concat(d->a3b, d->s2, n, d->H >> 3, d->W >> 3, 256, 128, d->cat2, s));
   TRY(c(8, d->cat2, d->u2a));
   TRY(c(9, d->u2a, d->u2b));
-  TRY(nn::up_fwd(d->u2b, n, d->H >> 2, d->W >> 2, 128, d->cat1, 192, 0, s));
-  TRY(nn::copy_channels(d->s1, npix(d, n, 1), 64, d->cat1, 192, 128, s));
+  TRY(nn::up_concat(d->u2b, d->s1, n, d->H >> 2, d->W >> 2, 128, 64, d->cat1, s));
   TRY(c(10, d->cat1, d->u1a));
   TRY(c(11, d->u1a, d->u1b));
-  TRY(nn::up_fwd(d->u1b, n, d->H >> 1, d->W >> 1, 64, d->cat0, 96, 0, s));
-  TRY(nn::copy_channels(d->s0, npix(d, n, 0), 32, d->cat0, 96, 64, s));
+  TRY(nn::up_concat(d->u1b, d->s0, n, d->H >> 1, d->W >> 1, 64, 32, d->cat0, s));
   TRY(c(12, d->cat0, d->u0a));
   TRY(c(13, d->u0a, d->u0b));
   TRY(c(14, d->u0b, d->out, true));
   return cudaSuccess;
 }
 
-// Backward through layer i: gradient g_y (FP32) at its output y (BF16, ReLU
-// mask when the layer has one), input x.  Accumulates the weight and bias
-// gradients; writes the input gradient into gx (rows [0, split)) and gx2
-// (rows [split, cin)) when those are non-null.
-cudaError_t back(Denoiser* d, int i, int n, const __nv_bfloat16* x, const __nv_bfloat16* y, const float* g_y, float* gx,
-                 float* gx2, int split, cudaStream_t s) {
+// Backward through layer i whose output gradient, masked and in BF16, is in
+// gbuf (its bias gradient is done): accumulates the weight gradient for the
+// input x; writes the input gradient into gx (rows [0, split)) and gx2 (rows
+// [split, cin)) when those are non-null.
+cudaError_t back_conv(Denoiser* d, int i, int n, const __nv_bfloat16* x, float* gx, float* gx2, int split,
+                      cudaStream_t s) {
   cudaError_t e;
   Layer& l = d->L[i];
   const int lev = kLevel[i];
   const size_t np = npix(d, n, lev);
-  TRY(nn::relu_mask(g_y, l.relu ? y : nullptr, np * l.cout, d->gbuf, s));
-  TRY(nn::bias_grad(d->gbuf, np, l.cout, l.gb, s));
   WgradParams wp;
   wp.x = x;
   wp.dy = d->gbuf;
@@ -183,30 +180,37 @@ cudaError_t back(Denoiser* d, int i, int n, const __nv_bfloat16* x, const __nv_b
   return cudaSuccess;
 }
 
+// The same from the gradient g of what the next stages made of the output y
+// (mode and gp: nn::mask).
+cudaError_t back(Denoiser* d, int i, int n, const __nv_bfloat16* x, const __nv_bfloat16* y, nn::MaskMode mode,
+                 const float* g, const float* gp, float* gx, float* gx2, int split, cudaStream_t s) {
+  cudaError_t e;
+  const int lev = kLevel[i];
+  TRY(nn::mask(mode, g, gp, y, n, d->H >> lev, d->W >> lev, d->L[i].cout, d->gbuf, d->L[i].gb, s));
+  return back_conv(d, i, n, x, gx, gx2, split, s);
+}
+
+// Backward pass from the output gradient in gbuf.
 cudaError_t backward(Denoiser* d, int n, cudaStream_t s) {
   cudaError_t e;
-  const int H = d->H, W = d->W;
-  TRY(back(d, 14, n, d->u0b, nullptr, d->g_out, d->g_u0b, nullptr, 0, s));
-  TRY(back(d, 13, n, d->u0a, d->u0b, d->g_u0b, d->g_u0a, nullptr, 0, s));
-  TRY(back(d, 12, n, d->cat0, d->u0a, d->g_u0a, d->g_cat0up, d->g_s0, 64, s));
-  TRY(nn::up_bwd(d->g_cat0up, n, H >> 1, W >> 1, 64, 64, 0, d->g_u1b, s));
-  TRY(back(d, 11, n, d->u1a, d->u1b, d->g_u1b, d->g_u1a, nullptr, 0, s));
-  TRY(back(d, 10, n, d->cat1, d->u1a, d->g_u1a, d->g_cat1up, d->g_s1, 128, s));
-  TRY(nn::up_bwd(d->g_cat1up, n, H >> 2, W >> 2, 128, 128, 0, d->g_u2b, s));
-  TRY(back(d, 9, n, d->u2a, d->u2b, d->g_u2b, d->g_u2a, nullptr, 0, s));
-  TRY(back(d, 8, n, d->cat2, d->u2a, d->g_u2a, d->g_cat2up, d->g_s2, 256, s));
-  TRY(nn::up_bwd(d->g_cat2up, n, H >> 3, W >> 3, 256, 256, 0, d->g_a3b, s));
-  TRY(back(d, 7, n, d->a3a, d->a3b, d->g_a3b, d->g_a3a, nullptr, 0, s));
-  TRY(back(d, 6, n, d->p2, d->a3a, d->g_a3a, d->g_p2, nullptr, 0, s));
-  TRY(nn::pool_bwd(d->s2, d->g_p2, n, H >> 2, W >> 2, 128, d->g_s2, s));
-  TRY(back(d, 5, n, d->a2a, d->s2, d->g_s2, d->g_a2a, nullptr, 0, s));
-  TRY(back(d, 4, n, d->p1, d->a2a, d->g_a2a, d->g_p1, nullptr, 0, s));
-  TRY(nn::pool_bwd(d->s1, d->g_p1, n, H >> 1, W >> 1, 64, d->g_s1, s));
-  TRY(back(d, 3, n, d->a1a, d->s1, d->g_s1, d->g_a1a, nullptr, 0, s));
-  TRY(back(d, 2, n, d->p0, d->a1a, d->g_a1a, d->g_p0, nullptr, 0, s));
-  TRY(nn::pool_bwd(d->s0, d->g_p0, n, H, W, 32, d->g_s0, s));
-  TRY(back(d, 1, n, d->a0a, d->s0, d->g_s0, d->g_a0a, nullptr, 0, s));
-  TRY(back(d, 0, n, d->in0, d->a0a, d->g_a0a, nullptr, nullptr, 0, s));
+  using nn::MASK_PLAIN;
+  using nn::MASK_POOL;
+  using nn::MASK_UP;
+  TRY(back_conv(d, 14, n, d->u0b, d->g_u0b, nullptr, 0, s));
+  TRY(back(d, 13, n, d->u0a, d->u0b, MASK_PLAIN, d->g_u0b, nullptr, d->g_u0a, nullptr, 0, s));
+  TRY(back(d, 12, n, d->cat0, d->u0a, MASK_PLAIN, d->g_u0a, nullptr, d->g_cat0up, d->g_s0, 64, s));
+  TRY(back(d, 11, n, d->u1a, d->u1b, MASK_UP, d->g_cat0up, nullptr, d->g_u1a, nullptr, 0, s));
+  TRY(back(d, 10, n, d->cat1, d->u1a, MASK_PLAIN, d->g_u1a, nullptr, d->g_cat1up, d->g_s1, 128, s));
+  TRY(back(d, 9, n, d->u2a, d->u2b, MASK_UP, d->g_cat1up, nullptr, d->g_u2a, nullptr, 0, s));
+  TRY(back(d, 8, n, d->cat2, d->u2a, MASK_PLAIN, d->g_u2a, nullptr, d->g_cat2up, d->g_s2, 256, s));
+  TRY(back(d, 7, n, d->a3a, d->a3b, MASK_UP, d->g_cat2up, nullptr, d->g_a3a, nullptr, 0, s));
+  TRY(back(d, 6, n, d->p2, d->a3a, MASK_PLAIN, d->g_a3a, nullptr, d->g_p2, nullptr, 0, s));
+  TRY(back(d, 5, n, d->a2a, d->s2, MASK_POOL, d->g_s2, d->g_p2, d->g_a2a, nullptr, 0, s));
+  TRY(back(d, 4, n, d->p1, d->a2a, MASK_PLAIN, d->g_a2a, nullptr, d->g_p1, nullptr, 0, s));
+  TRY(back(d, 3, n, d->a1a, d->s1, MASK_POOL, d->g_s1, d->g_p1, d->g_a1a, nullptr, 0, s));
+  TRY(back(d, 2, n, d->p0, d->a1a, MASK_PLAIN, d->g_a1a, nullptr, d->g_p0, nullptr, 0, s));
+  TRY(back(d, 1, n, d->a0a, d->s0, MASK_POOL, d->g_s0, d->g_p0, d->g_a0a, nullptr, 0, s));
+  TRY(back(d, 0, n, d->in0, d->a0a, MASK_PLAIN, d->g_a0a, nullptr, nullptr, nullptr, 0, s));
   return cudaSuccess;
 }
 
@@ -251,14 +255,24 @@ cudaError_t denoiser_create(int H, int W, int B, unsigned long long seed, Denois
   A(d->stage_in, n0);
   A(d->stage_out, n0);
   A(d->gbuf, std::max(std::max(n0 * 32, n1 * 64), std::max(n2 * 128, n3 * 256)));
-  A(d->g_out, n0 * 16); A(d->g_u0b, n0 * 32); A(d->g_u0a, n0 * 32); A(d->g_cat0up, n0 * 64); A(d->g_s0, n0 * 32);
-  A(d->g_u1b, n1 * 64); A(d->g_u1a, n1 * 64); A(d->g_cat1up, n1 * 128); A(d->g_s1, n1 * 64);
-  A(d->g_u2b, n2 * 128); A(d->g_u2a, n2 * 128); A(d->g_cat2up, n2 * 256); A(d->g_s2, n2 * 128);
-  A(d->g_a3b, n3 * 256); A(d->g_a3a, n3 * 256); A(d->g_p2, n3 * 128);
+  A(d->g_u0b, n0 * 32); A(d->g_u0a, n0 * 32); A(d->g_cat0up, n0 * 64); A(d->g_s0, n0 * 32);
+  A(d->g_u1a, n1 * 64); A(d->g_cat1up, n1 * 128); A(d->g_s1, n1 * 64);
+  A(d->g_u2a, n2 * 128); A(d->g_cat2up, n2 * 256); A(d->g_s2, n2 * 128);
+  A(d->g_a3a, n3 * 256); A(d->g_p2, n3 * 128);
   A(d->g_a2a, n2 * 128); A(d->g_p1, n2 * 64); A(d->g_a1a, n1 * 64); A(d->g_p0, n1 * 32); A(d->g_a0a, n0 * 32);
   A(d->scale, (size_t)B);
   A(d->loss, (size_t)1);
   A(d->err, (size_t)1);
+  d->table.layers = kLayers;
+  uint32_t total = 0;
+  for (int i = 0; i < kLayers; ++i) {
+    d->table.begin[i] = total;
+    d->table.cin[i] = kCin[i];
+    d->table.cout[i] = kCout[i];
+    total += (uint32_t)(kCout[i] * 9 * kCin[i] + kCout[i]);
+  }
+  d->table.begin[kLayers] = total;
+  A(d->par, (size_t)total); A(d->grad, (size_t)total); A(d->mom, (size_t)total); A(d->var, (size_t)total);
   std::mt19937_64 rng(seed);
   std::normal_distribution<float> nd(0.f, 1.f);
   for (int i = 0; i < kLayers && e == cudaSuccess; ++i) {
@@ -267,9 +281,14 @@ cudaError_t denoiser_create(int H, int W, int B, unsigned long long seed, Denois
     l.cout = kCout[i];
     l.relu = i != kLayers - 1;
     const size_t nw = l.nw();
-    A(l.w, nw); A(l.gw, nw); A(l.mw, nw); A(l.vw, nw); A(l.wb, nw); A(l.wt, nw);
-    A(l.b, (size_t)l.cout); A(l.gb, (size_t)l.cout); A(l.mb, (size_t)l.cout); A(l.vb, (size_t)l.cout);
+    A(l.wb, nw); A(l.wt, nw);
     if (e != cudaSuccess) break;
+    l.w = d->par + d->table.begin[i];
+    l.b = l.w + nw;
+    l.gw = d->grad + d->table.begin[i];
+    l.gb = l.gw + nw;
+    d->table.wf[i] = l.wb;
+    d->table.wa[i] = l.wt;
     // He initialisation over the real fan-in (the first layer sees one channel);
     // the output layer starts small so the initial residual is close to zero
     const int fan_in = 9 * (i == 0 ? 1 : l.cin);
@@ -344,20 +363,11 @@ cudaError_t denoiser_train_step(Denoiser* d, const float* noisy, const float* cl
   TRY(cudaMemsetAsync(d->loss, 0, 8, s));
   TRY(cudaMemsetAsync(d->err, 0, 4, s));
   TRY(forward(d, noisy, n, s));
-  TRY(nn::mse(noisy, clean, d->scale, d->out, n, d->H * d->W, d->g_out, d->loss, s));
-  for (auto& l : d->L) {
-    TRY(cudaMemsetAsync(l.gw, 0, l.nw() * 4, s));
-    TRY(cudaMemsetAsync(l.gb, 0, (size_t)l.cout * 4, s));
-  }
+  TRY(cudaMemsetAsync(d->grad, 0, (size_t)d->table.begin[kLayers] * 4, s));
+  TRY(nn::mse(noisy, clean, d->scale, d->out, n, d->H * d->W, d->gbuf, d->L[14].gb, d->loss, s));
   TRY(backward(d, n, s));
   d->step += 1;
-  if (lr > 0.f) {
-    for (auto& l : d->L) {
-      TRY(nn::adam(l.w, l.gw, l.mw, l.vw, l.nw(), lr, d->step, nullptr, s));
-      TRY(nn::adam(l.b, l.gb, l.mb, l.vb, (size_t)l.cout, lr, d->step, nullptr, s));
-      TRY(nn::pack_weights(l.w, l.cout, l.cin, l.wb, l.wt, s));
-    }
-  }
+  if (lr > 0.f) TRY(nn::adam(d->par, d->grad, d->mom, d->var, d->table, lr, d->step, s));
   double loss = 0;
   TRY(cudaMemcpyAsync(&loss, d->loss, 8, cudaMemcpyDeviceToHost, s));
   TRY(cudaMemcpyAsync(err_out, d->err, 4, cudaMemcpyDeviceToHost, s));
