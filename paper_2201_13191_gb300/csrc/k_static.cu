@@ -220,14 +220,12 @@ extern "C" int mc_project_scatter_static(mc_ctx* ctx, const float* angles_rad, i
   const int smem = transport_smem_bytes(tv, nb, block);
   int per_sm = opt.blocks_per_sm;
   if (per_sm == 0) {
-    e = transport_occupancy(block, smem, &per_sm, false, vv.layout);
+    e = transport_occupancy(block, smem, &per_sm, false, vv.layout, !opt.nee_mode && !opt.doppler, vv.words);
     if (e != cudaSuccess) return static_cuda_fail(ctx, e, "occupancy query");
     per_sm = per_sm > 0 ? per_sm : 1;
   }
   const unsigned long long work = (unsigned long long)n_angles * n_photons;
-  const unsigned long long need = (work + block - 1) / block;
-  const unsigned long long cap = (unsigned long long)sm_count * per_sm;
-  const int grid = (int)(need < cap ? (need > 0 ? need : 1) : cap);
+  const int grid = transport_grid(work, block, sm_count * per_sm, vv.layout, true, &tp.hist_chunk);
   e = launch_transport(tp, grid, block, s);
   if (e == cudaSuccess) e = launch_finalize(tally, 1, n_img, scatter_out, nullptr, s);
   if (e != cudaSuccess) return static_cuda_fail(ctx, e, "static transport launch");

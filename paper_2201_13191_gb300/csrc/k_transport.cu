@@ -131,6 +131,39 @@ __device__ __forceinline__ float3 hop_point(const VoxRay& r, float k, float h, f
                      fmaf(u, hv.z, fmaf(t0, r.vw.z, r.v0.z)));
 }
 
+// A flight's m steps through one material of attenuation mu (mm^-1), h mm each:
+// adds their optical depths to tau and returns false, or, if a step's end reaches
+// tau_star, leaves tau at that step's start, its number in ks, and returns true.
+//
+// tau takes the FP32 sums of the step-by-step march, rounding for rounding, so
+// the interaction points are the same, but most of them are not formed: while the
+// sum stays in one binade every addition of the same term adds the same multiple
+// q of its unit in the last place (a tie goes to even; the sum after one is even,
+// and the next additions repeat), hence j additions add exactly j q.  Three steps
+// are taken one by one, the rest at once up to the binade's end or two steps
+// short of tau_star: 0.04 rounds per step over a flight's words.
+__device__ __forceinline__ bool flight_word(float mu, float h, float tau_star, float m, float& tau, float& ks) {
+  float left = m;
+  do {
+    const float t1 = fmaf(mu, h, tau), t2 = fmaf(mu, h, t1), t3 = fmaf(mu, h, t2);
+    const float end = left < 2.f ? t1 : left < 3.f ? t2 : t3;
+    if (end >= tau_star) {
+      ks = m - left + (t1 >= tau_star ? 0.f : t2 >= tau_star ? 1.f : 2.f);
+      tau = t1 >= tau_star ? tau : t2 >= tau_star ? t1 : t2;
+      return true;
+    }
+    const float q = t3 - t2;
+    const uint32_t e3 = __float_as_uint(t3) & 0x7F800000u;
+    const float top = __uint_as_float(e3 + 0x00800000u);
+    float j = __fadd_rd(__fdividef(fminf(top, tau_star) - t3, q), 8388608.f) - 8388610.f;
+    if ((__float_as_uint(t1) & 0x7F800000u) != e3) j = 0.f;
+    j = fmaxf(q > 0.f ? fminf(j, left - 3.f) : left - 3.f, 0.f);
+    tau = left > 3.f ? fmaf(j, q, t3) : end;
+    left -= 3.f + j;
+  } while (left > 0.f);
+  return false;
+}
+
 // Adds the group's steps to the optical-depth sum acc (attenuation per unit
 // density from this thread's shared-memory column smu); TAIL masks the steps
 // k0 + u >= n.
@@ -649,24 +682,20 @@ __device__ __forceinline__ void pseudo_particle(const TransportParams& P, const 
   tally_add<COMBINE>(P, s_img, off, x0 * __expf(-tp));
 }
 
-#ifndef MC_MIN_BLOCKS
-#define MC_MIN_BLOCKS 2
-#endif
-// The same for the brick layout (volumes in HBM, where more warps in flight hide
-// the longer gathers).
-#ifndef MC_MIN_BLOCKS_BRICK
-#define MC_MIN_BLOCKS_BRICK MC_MIN_BLOCKS
-#endif
+// Blocks of 256 threads per SM that a variant's registers must leave room for.
+// A march through a volume with clearance is a chain of dependent gathers, so
+// more warps pay even for a few spilled registers: 256^3 ellipsoids, 2e7 photons
+// 33.8 / 30.9 / 32.6 ms with 2 / 3 / 4 blocks, 512^3 (its words in HBM), 6 x 8e5
+// photons 13.5 / 10.4 / 9.2 ms.  The step-by-step marches keep the L1 data pipe
+// busy with 2, and the expected-value and Doppler forms spill too much beyond 2.
+constexpr int min_blocks(int layout, bool combine, bool ev, bool dop, bool hbm) {
+  return layout == VOX_HOP && !combine && !ev && !dop ? (hbm ? 4 : 3) : 2;
+}
 // Flights through a linear-layout volume sum each group's optical depth
 // branch-free before looking for the interaction step (1), or test every step
 // (0); both give the same interaction points.
 #ifndef MC_FLIGHT_GROUP
 #define MC_FLIGHT_GROUP 1
-#endif
-// Flights per lane and iteration with the per-warp phases (the block-wide
-// phases of the combined tallies take one).
-#ifndef MC_FLIGHTS_PER_ITER
-#define MC_FLIGHTS_PER_ITER 1
 #endif
 // Pseudo-particle jobs are handed out longest records first: records are
 // bucketed by the chord from the interaction point to the volume boundary
@@ -722,9 +751,8 @@ __device__ void tile_fetch(const TransportParams& P, uint2 key, TileChunk& c) {
   }
 }
 
-template <int LAYOUT, bool COMBINE, bool EV, bool DOP>
-__global__ void __launch_bounds__(256, LAYOUT == VOX_BRICK ? MC_MIN_BLOCKS_BRICK : MC_MIN_BLOCKS)
-    k_transport(const TransportParams P) {
+template <int LAYOUT, bool COMBINE, bool EV, bool DOP, int MINB>
+__global__ void __launch_bounds__(256, MINB) k_transport(const TransportParams P) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ uint64_t bar;
   __shared__ int s_nrec, s_job;
@@ -739,7 +767,6 @@ __global__ void __launch_bounds__(256, LAYOUT == VOX_BRICK ? MC_MIN_BLOCKS_BRICK
   // in HBM (brick layout), where they were measured faster than per-warp
   // phases; per-warp phases otherwise.
   constexpr bool kBlockPhases = COMBINE || LAYOUT == VOX_BRICK;
-  constexpr int kFlights = kBlockPhases ? 1 : MC_FLIGHTS_PER_ITER;
   const int nm = P.tab.n_mat, ns = P.tab.n_stage;
   const int nb = P.spec.n_bins;
   const int B = blockDim.x;
@@ -825,6 +852,11 @@ __global__ void __launch_bounds__(256, LAYOUT == VOX_BRICK ? MC_MIN_BLOCKS_BRICK
   const unsigned long long total = (unsigned long long)P.n_angles * P.h_count;
   const unsigned long long stride = (unsigned long long)gridDim.x * B;
   unsigned long long next = (unsigned long long)blockIdx.x * B + threadIdx.x;
+  // Per-warp phases take their histories from a global counter, hist_chunk at a time, so that no warp is left with
+  // more work than the others at the end (a fixed share each: 256^3 ellipsoids 30.9 -> 28.8 ms, triangle meshes 14.9
+  // -> 12.5); [w_next, w_end) is the warp's reserve.
+  unsigned long long w_next = 0, w_end = 0;
+  bool w_more = !kBlockPhases;
 
   // photon state
   bool alive = false;
@@ -844,13 +876,37 @@ __global__ void __launch_bounds__(256, LAYOUT == VOX_BRICK ? MC_MIN_BLOCKS_BRICK
 
   for (;;) {
     if (tiled && s_tc.done) break;
-    // ---- flight phase: one free flight per live photon; with the per-warp
-    // phases a lane whose photon leaves without a record (escape, absorption)
-    // starts the next history in the same iteration, up to kFlights flights
+    // ---- flight phase: one free flight per live photon
     bool has_rec = false;
-    for (int fl = 0; fl < kFlights; ++fl) {
+    {
       bool fresh = false;
-      if (tiled) {
+      if constexpr (!kBlockPhases) {
+        // idle lanes take the rest of the warp's reserve, then of the next one
+        const unsigned need = __ballot_sync(0xffffffffu, !alive);
+        const unsigned long long want = (unsigned long long)__popc(need), left = w_end - w_next;
+        const unsigned long long mine = (unsigned long long)__popc(need & ((1u << (threadIdx.x & 31)) - 1u));
+        unsigned long long idx = w_next + mine;
+        bool has = mine < left;
+        if (want > left && w_more) {
+          unsigned long long base = 0;
+          if ((threadIdx.x & 31) == 0) base = atomicAdd(P.stats + S_WORK, (unsigned long long)P.hist_chunk);
+          base = __shfl_sync(0xffffffffu, base, 0);
+          w_more = base < total;
+          w_end = w_more ? min(base + (unsigned long long)P.hist_chunk, total) : base;
+          w_next = min(base + (want - left), w_end);
+          if (!has) {
+            idx = base + (mine - left);
+            has = idx < w_end;
+          }
+        } else {
+          w_next = min(w_next + want, w_end);
+        }
+        if (!alive && has) {
+          a = (int)(idx / P.h_count);
+          h = P.h_begin + (idx - (unsigned long long)a * P.h_count);
+          fresh = true;
+        }
+      } else if (tiled) {
         if (!alive) {
           const unsigned long long j = atomicAdd(&s_tc.j, 1ull);
           if (j < s_tc.j_end) {
@@ -963,43 +1019,25 @@ __global__ void __launch_bounds__(256, LAYOUT == VOX_BRICK ? MC_MIN_BLOCKS_BRICK
           };
           int k0 = 0;
           if constexpr (LAYOUT == VOX_HOP) {
-            // one word stands for its clearance's steps; their optical depths are added one by one, in the
-            // order and with the roundings of the step-by-step march, so the interaction points are the same
+            // one word stands for the steps in its uniform cube (flight_word)
             Hop hop;
             hop.set(vr, hv, (float)n);
             const float nf = (float)n;
-            float kn = 0.f, left = 0.f, mu = 0.f;  // next step to load, steps left of the current word
-            for (;;) {
-              if (left <= 0.f) {
-                if (kn >= nf) break;
-                const float3 p = hop_point(vr, kn, hh, ta, hv);
-                const uint32_t hw = __ldg(V.vox + vr.voxel_p<LAYOUT>(V, p.x, p.y, p.z));
-                left = fminf(hop.steps(hw, p), nf - kn);
-                const uint32_t wd = T.pal[hw & 255u];
-                cur = vox_mat(wd);
-                mu = my_mu[cur * B] * vox_rho(wd);
-                kn += left;
-              }
-              float t = tau;
-#pragma unroll
-              for (int u = 0; u < kLook; ++u) t = (float)u < left ? fmaf(mu, hh, t) : t;
-              if (t >= tau_star) {
-                // the step whose end reaches tau* holds the interaction
-                float ks = kn - left;
-                for (;;) {
-                  t = fmaf(mu, hh, tau);
-                  if (t >= tau_star) break;
-                  tau = t;
-                  ks += 1.f;
-                }
+            for (float kn = 0.f; kn < nf && !hit;) {
+              const float3 p = hop_point(vr, kn, hh, ta, hv);
+              const uint32_t hw = __ldg(V.vox + vr.voxel_p<LAYOUT>(V, p.x, p.y, p.z));
+              const float m = fminf(hop.steps(hw, p), nf - kn);
+              const uint32_t wd = T.pal[hw & 255u];
+              const float mu = my_mu[vox_mat(wd) * B] * vox_rho(wd);
+              float ks;
+              if (flight_word(mu, hh, tau_star, m, tau, ks)) {
+                ks += kn;
                 tint = fmaf(ks, hh, ta) + (tau_star - tau) / mu;
-                mint = cur;
+                mint = vox_mat(wd);
                 hit = true;
                 k = (int)ks;
-                break;
               }
-              tau = t;
-              left -= (float)kLook;
+              kn += m;
             }
           }
           if (LAYOUT == VOX_BRICK && MC_BRICK_NOSPLIT) {
@@ -1108,7 +1146,6 @@ __global__ void __launch_bounds__(256, LAYOUT == VOX_BRICK ? MC_MIN_BLOCKS_BRICK
           }
         }
       }
-      if (has_rec || !(alive || next < total)) break;
     }
     if constexpr (!kBlockPhases) {
       // ---- pseudo-particle phase, per warp (no block barrier): the warp marches
@@ -1139,7 +1176,7 @@ __global__ void __launch_bounds__(256, LAYOUT == VOX_BRICK ? MC_MIN_BLOCKS_BRICK
       }
       // every lane has read the warp's records before they are overwritten
       __syncwarp();
-      if (!__any_sync(0xffffffffu, alive || next < total)) break;
+      if (!__any_sync(0xffffffffu, alive) && !w_more && w_next >= w_end) break;
       continue;
     }
     __syncthreads();
@@ -1270,23 +1307,44 @@ int transport_smem_bytes(const TableView& t, int n_bins, int block, int shared_p
 }
 
 namespace {
-template <int LAYOUT, bool COMBINE, bool EV, bool DOP>
+template <int LAYOUT, bool COMBINE, bool EV, bool DOP, bool HBM = false>
 cudaError_t launch_one(const TransportParams& p, int grid, int block, int smem, cudaStream_t s) {
-  cudaError_t e = cudaFuncSetAttribute(k_transport<LAYOUT, COMBINE, EV, DOP>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  auto* k = k_transport<LAYOUT, COMBINE, EV, DOP, min_blocks(LAYOUT, COMBINE, EV, DOP, HBM)>;
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  k_transport<LAYOUT, COMBINE, EV, DOP><<<grid, block, smem, s>>>(p);
+  k<<<grid, block, smem, s>>>(p);
   return cudaGetLastError();
 }
+
+// A packed volume beyond 3/4 of the 126 MB L2 streams from HBM (the line at which the layouts change, too).
+constexpr long long kL2Words = (long long)(0.75 * 126e6) / 4;
 }  // namespace
 
-cudaError_t transport_occupancy(int block, int smem, int* blocks_per_sm, bool mesh, int layout) {
-  auto* k = mesh                    ? k_transport<GEO_MESH, false, false, false>
-            : layout == VOX_BRICK ? k_transport<VOX_BRICK, false, false, false>
-            : layout == VOX_HOP   ? k_transport<VOX_HOP, false, false, false>
-                                  : k_transport<VOX_LIN, false, false, false>;
+cudaError_t transport_occupancy(int block, int smem, int* blocks_per_sm, bool mesh, int layout, bool plain, int words) {
+  const bool hbm = words > kL2Words;
+  auto* k = mesh                  ? k_transport<GEO_MESH, false, false, false, 2>
+            : layout == VOX_BRICK ? k_transport<VOX_BRICK, false, false, false, 2>
+            : layout != VOX_HOP   ? k_transport<VOX_LIN, false, false, false, 2>
+            : !plain              ? k_transport<VOX_HOP, false, true, true, 2>
+            : hbm ? k_transport<VOX_HOP, false, false, false, min_blocks(VOX_HOP, false, false, false, true)>
+                  : k_transport<VOX_HOP, false, false, false, min_blocks(VOX_HOP, false, false, false, false)>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, block, smem);
+}
+
+int transport_grid(unsigned long long work, int block, int room, int layout, bool global_tally, int* hist_chunk) {
+  *hist_chunk = 32;
+  if (work == 0) return 0;
+  // Per-warp phases: few histories are spread over all the SMs' warps, since a warp with few photons finishes sooner
+  // (2e4 histories of an 8^3 phantom: 79 blocks of full warps 0.090 ms, a few photons per warp 0.080).
+  // The block-wide phases fill their blocks.
+  const bool per_warp = global_tally && layout != VOX_BRICK;
+  const unsigned long long per_block = per_warp ? (unsigned long long)(block / 32) : (unsigned long long)block;
+  const int grid = (int)std::min<unsigned long long>((work + per_block - 1) / per_block, (unsigned long long)std::max(room, 1));
+  const unsigned long long warps = (unsigned long long)grid * (block / 32);
+  *hist_chunk = (int)std::min<unsigned long long>(32, std::max<unsigned long long>(1, (work + warps - 1) / warps));
+  return grid;
 }
 
 cudaError_t launch_transport(const TransportParams& p, int grid, int block, cudaStream_t s) {
@@ -1321,7 +1379,9 @@ cudaError_t launch_transport(const TransportParams& p, int grid, int block, cuda
     MC_LAUNCH(17, GEO_MESH, false, false, true)
     MC_LAUNCH(18, GEO_MESH, false, true, false)
     MC_LAUNCH(19, GEO_MESH, false, true, true)
-    MC_LAUNCH(24, VOX_HOP, false, false, false)
+    case 24:
+      return p.vol.words > kL2Words ? launch_one<VOX_HOP, false, false, false, true>(p, grid, block, smem, s)
+                                    : launch_one<VOX_HOP, false, false, false>(p, grid, block, smem, s);
     MC_LAUNCH(25, VOX_HOP, false, false, true)
     MC_LAUNCH(26, VOX_HOP, false, true, false)
     MC_LAUNCH(27, VOX_HOP, false, true, true)

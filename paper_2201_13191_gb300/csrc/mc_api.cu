@@ -520,13 +520,14 @@ int project_impl(mc_ctx* ctx, const float* angles, int n_angles, uint64_t N, uin
     const int smem = transport_smem_bytes(tp.tab, sv.n_bins, block, transport_shared_pixels(tp));
     int per_sm = ctx->opt.blocks_per_sm;
     if (per_sm == 0) {
-      CK(transport_occupancy(block, smem, &per_sm, ctx->mesh_mode, ctx->layout), "occupancy query");
+      CK(transport_occupancy(block, smem, &per_sm, ctx->mesh_mode, ctx->layout,
+                             !tp.nee_mode && !tp.doppler && tp.tally_mode == TALLY_GLOBAL, tp.vol.words),
+         "occupancy query");
       per_sm = std::max(1, per_sm);
     }
     const unsigned long long work = (unsigned long long)n_angles * h_count;
-    const unsigned long long need = (work + block - 1) / block;
-    grid = (int)std::max<unsigned long long>(1, std::min<unsigned long long>(need, (unsigned long long)ctx->sm_count * per_sm));
-    if (work == 0) grid = 0;
+    grid = transport_grid(work, block, ctx->sm_count * per_sm, ctx->mesh_mode ? GEO_MESH : ctx->layout,
+                          ctx->mesh_mode || tp.tally_mode == TALLY_GLOBAL, &tp.hist_chunk);
     if (tp.tally_mode == TALLY_TILED && grid > 0) {
       // chunks of one (angle, tile): about 8 per block for balance, at least 4 histories per thread so
       // that the wait for a chunk's last photon stays short, at most a tile's share of the run
@@ -1111,11 +1112,13 @@ int mc_autotune(mc_ctx* ctx, const float* angles, int n_angles, uint64_t probe, 
   }
   // 2. launch shape at the chosen step
   const mc_options saved = ctx->opt;
+  const bool plain = !ctx->opt.nee_mode && !ctx->opt.doppler;
+  const int words = volume_view(ctx).words;
   int smem = 0, max_per_sm = 1;
   {
     const TableView tv = table_view(ctx);
     smem = transport_smem_bytes(tv, (int)ctx->S.size(), 256, 0);
-    e = transport_occupancy(256, smem, &max_per_sm, ctx->mesh_mode, ctx->layout);
+    e = transport_occupancy(256, smem, &max_per_sm, false, ctx->layout, plain, words);
     if (e != cudaSuccess) return finish(cuda_fail(ctx, e, "occupancy query"));
   }
   double best_rate = -1;
@@ -1125,7 +1128,7 @@ int mc_autotune(mc_ctx* ctx, const float* angles, int n_angles, uint64_t probe, 
   for (int bi = 0; bi < 3; ++bi) {
     int occ = 1;
     e = transport_occupancy(blocks[bi], transport_smem_bytes(table_view(ctx), (int)ctx->S.size(), blocks[bi], 0), &occ,
-                            ctx->mesh_mode, ctx->layout);
+                            false, ctx->layout, plain, words);
     if (e != cudaSuccess) return finish(cuda_fail(ctx, e, "occupancy query"));
     for (int per = 1; per <= std::max(1, occ); ++per) {
       for (int ti = 0; ti < 2; ++ti) {

@@ -125,6 +125,7 @@ struct TransportParams {
   // half extents of a box around the bodies (hx, hy, hz)
   int geometry = 0;  // VOX_* from vol.layout, or GEO_MESH
   MeshView mesh = {};
+  int hist_chunk = 32;  // histories a warp reserves at a time (kernels with per-warp phases)
   // TALLY_TILED: tiles of tile_u x tile_v pixels, n_tu across, n_tiles in all;
   // work in chunks of up to tile_chunk histories of one (angle, tile), tile_k
   // chunks per (angle, tile), n_chunks in all, handed out by stats[S_WORK]
@@ -163,7 +164,11 @@ cudaError_t launch_transport(const TransportParams& p, int grid, int block, cuda
 int transport_smem_bytes(const TableView& t, int n_bins, int block, int shared_pixels = 0);
 // FP32 pixels of the shared tally image the kernel keeps for these parameters
 int transport_shared_pixels(const TransportParams& p);
-cudaError_t transport_occupancy(int block, int smem, int* blocks_per_sm, bool mesh = false, int layout = VOX_LIN);
+// plain: sampled-type scores without Doppler broadening, global tally; words: the packed volume's
+cudaError_t transport_occupancy(int block, int smem, int* blocks_per_sm, bool mesh, int layout, bool plain, int words);
+// Blocks of a launch of `work` histories (at least one if there are any; at most `room`), and the histories a warp
+// reserves at a time.
+int transport_grid(unsigned long long work, int block, int room, int layout, bool global_tally, int* hist_chunk);
 cudaError_t launch_finalize(const double* tally, int n_batches, size_t n, float* out, float* var, cudaStream_t s);
 cudaError_t launch_primary(const PrimaryParams& p, cudaStream_t s);
 
