@@ -229,119 +229,199 @@ cudaError_t filter_direct(const float* p, int nu, int nv, int rows_total, float 
   return cudaGetLastError();
 }
 
-// Histogram of vol over [lo, hi) in nbins bins (values outside are clamped to the end bins).
-__global__ void k_hist(const float* __restrict__ vol, size_t n, float lo, float hi, int nbins,
-                       unsigned int* __restrict__ hist) {
-  extern __shared__ unsigned int sh[];
-  for (int b = threadIdx.x; b < nbins; b += blockDim.x) sh[b] = 0;
+constexpr int kBins = 256;
+
+__device__ __forceinline__ int bin_of(float v, float lo, float sc) {
+  return min(max((int)((v - lo) * sc), 0), kBins - 1);
+}
+
+// Histogram of vol over [lo, hi) in kBins bins (values outside are clamped to
+// the end bins).  A volume's voxels crowd a few bins (air, water), where one
+// shared counter per bin serialises a warp: each lane counts in its own copy
+// (copy = lane = bank).  256^3: 39 -> 18 us.
+__global__ void __launch_bounds__(256) k_hist(const float* __restrict__ vol, size_t n, float lo, float hi,
+                                              unsigned int* __restrict__ hist) {
+  __shared__ unsigned int sh[kBins * 32];
+  for (int b = threadIdx.x; b < kBins * 32; b += blockDim.x) sh[b] = 0;
   __syncthreads();
-  const float sc = (float)nbins / (hi - lo);
-  for (size_t i = gtid(); i < n; i += gstride()) {
-    const int b = min(max((int)((vol[i] - lo) * sc), 0), nbins - 1);
-    atomicAdd(&sh[b], 1u);
+  const int lane = threadIdx.x & 31;
+  const float sc = (float)kBins / (hi - lo);
+  const size_t n4 = ((uintptr_t)vol & 15) == 0 ? n / 4 : 0;
+  for (size_t i = gtid(); i < n4; i += gstride()) {
+    const float4 v = __ldg(reinterpret_cast<const float4*>(vol) + i);
+    atomicAdd(&sh[bin_of(v.x, lo, sc) * 32 + lane], 1u);
+    atomicAdd(&sh[bin_of(v.y, lo, sc) * 32 + lane], 1u);
+    atomicAdd(&sh[bin_of(v.z, lo, sc) * 32 + lane], 1u);
+    atomicAdd(&sh[bin_of(v.w, lo, sc) * 32 + lane], 1u);
   }
+  for (size_t i = 4 * n4 + gtid(); i < n; i += gstride()) atomicAdd(&sh[bin_of(vol[i], lo, sc) * 32 + lane], 1u);
   __syncthreads();
-  for (int b = threadIdx.x; b < nbins; b += blockDim.x)
-    if (sh[b]) atomicAdd(&hist[b], sh[b]);
+  for (int b = threadIdx.x; b < kBins; b += blockDim.x) {
+    unsigned int t = 0;
+    for (int k = 0; k < 32; ++k) t += sh[b * 32 + ((k + b) & 31)];
+    if (t) atomicAdd(&hist[b], t);
+  }
 }
 
 // Multi-level Otsu (classes = 2 or 3): thresholds maximising the between-class
-// variance of the histogram, exhaustively (one block; nbins <= 256).
-__global__ void k_otsu(const unsigned int* __restrict__ hist, int nbins, int classes, int* __restrict__ thr) {
-  __shared__ double P[257], S[257];
-  __shared__ double best_val[256];
-  __shared__ int best_a[256], best_b[256];
-  if (threadIdx.x == 0) {
-    P[0] = 0;
-    S[0] = 0;
-    for (int b = 0; b < nbins; ++b) {
-      P[b + 1] = P[b] + hist[b];
-      S[b + 1] = S[b] + (double)hist[b] * (b + 0.5);
-    }
-  }
+// variance of the histogram, exhaustively, ties to the smallest.  Bound by the
+// FP64 divisions of its 32640 candidates, two lanes a clock and SM: block a - 1
+// takes the candidates with first threshold a, thread b - 1 the second threshold
+// b, and the last block to finish picks the best (one block over all: 563 us).
+struct OtsuScratch {
+  double val[kBins];
+  int second[kBins];
+  unsigned int done;
+};
+__global__ void __launch_bounds__(kBins) k_otsu(const unsigned int* __restrict__ hist, int classes, OtsuScratch* sc,
+                                                int* __restrict__ thr) {
+  __shared__ double P[kBins + 1], S[kBins + 1];
+  __shared__ double val[kBins];
+  __shared__ int at[kBins];
+  __shared__ bool last;
+  const int t = threadIdx.x;
+  // counts and count-weighted bin centres are multiples of 1/2 below 2^52: their sums are exact in any order
+  if (t == 0) P[0] = S[0] = 0.0;
+  P[t + 1] = (double)hist[t];
+  S[t + 1] = (double)hist[t] * (t + 0.5);
   __syncthreads();
-  const double N = P[nbins], mu = S[nbins] / fmax(N, 1.0);
+  for (int o = 1; o < kBins; o <<= 1) {
+    const double p = t >= o ? P[t + 1 - o] : 0.0, s = t >= o ? S[t + 1 - o] : 0.0;
+    __syncthreads();
+    P[t + 1] += p;
+    S[t + 1] += s;
+    __syncthreads();
+  }
+  const double N = P[kBins], mu = S[kBins] / fmax(N, 1.0);
   auto term = [&](int a, int b) {  // class [a, b)
     const double w = P[b] - P[a];
     if (w <= 0) return 0.0;
     const double m = (S[b] - S[a]) / w;
     return w * (m - mu) * (m - mu);
   };
-  double bv = -1;
-  int ba = 1, bb = nbins;
-  for (int a = 1 + threadIdx.x; a < nbins; a += blockDim.x) {
-    if (classes == 2) {
-      const double v = term(0, a) + term(a, nbins);
-      if (v > bv) { bv = v; ba = a; bb = nbins; }
-    } else {
-      for (int b = a + 1; b < nbins; ++b) {
-        const double v = term(0, a) + term(a, b) + term(b, nbins);
-        if (v > bv) { bv = v; ba = a; bb = b; }
-      }
+  const int a = 1 + blockIdx.x;  // first threshold, 1 .. kBins - 1
+  double v = -1.0;
+  int b = kBins;
+  if (classes == 2) {
+    if (t == 0) v = term(0, a) + term(a, kBins);
+  } else {
+    const int bb = 1 + t;
+    if (bb > a && bb < kBins) {
+      v = term(0, a) + term(a, bb) + term(bb, kBins);
+      b = bb;
     }
   }
-  best_val[threadIdx.x] = bv;
-  best_a[threadIdx.x] = ba;
-  best_b[threadIdx.x] = bb;
+  val[t] = v;
+  at[t] = b;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    int k = 0;
-    for (int t = 1; t < (int)blockDim.x; ++t)
-      if (best_val[t] > best_val[k] || (best_val[t] == best_val[k] && (best_a[t] < best_a[k] ||
-                                                                     (best_a[t] == best_a[k] && best_b[t] < best_b[k]))))
-        k = t;
-    thr[0] = best_a[k];
-    thr[1] = best_b[k];
+  // largest value, the smallest index among equals
+  auto best = [&]() {
+    for (int o = kBins / 2; o > 0; o >>= 1) {
+      if (t < o && (val[t + o] > val[t] || (val[t + o] == val[t] && at[t + o] < at[t]))) {
+        val[t] = val[t + o];
+        at[t] = at[t + o];
+      }
+      __syncthreads();
+    }
+  };
+  best();
+  if (t == 0) {
+    sc->val[a] = val[0];
+    sc->second[a] = at[0];
+    __threadfence();
+    last = atomicAdd(&sc->done, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  val[t] = t >= 1 ? __ldcg(sc->val + t) : -2.0;
+  at[t] = t;
+  __syncthreads();
+  best();
+  if (t == 0) {
+    // without a candidate (no second threshold above the first): the first pair
+    thr[0] = val[0] >= 0.0 ? at[0] : 1;
+    thr[1] = val[0] >= 0.0 ? __ldcg(sc->second + at[0]) : kBins;
   }
 }
 
 // Class of each voxel by the thresholds (bins) -> material id and density
 // rho = mu / (mu_rho(material) * 0.1), clamped to [0, rho_max]; class 0 -> the
-// background material at its nominal density.
-__global__ void k_segment(const float* __restrict__ vol, size_t n, float lo, float hi, int nbins,
-                          const int* __restrict__ thr, int classes, const int* __restrict__ cls_mat,
-                          const float* __restrict__ cls_murho, const float* __restrict__ cls_rho0, float rho_max,
-                          uint8_t* __restrict__ mat, uint16_t* __restrict__ rho) {
-  const float sc = (float)nbins / (hi - lo);
+// background material at its nominal density.  Four voxels per thread where the
+// arrays are aligned for it.
+__global__ void __launch_bounds__(256) k_segment(const float* __restrict__ vol, size_t n, float lo, float hi,
+                                                 const int* __restrict__ thr, int classes, SegmentClasses cls,
+                                                 float rho_max, uint8_t* __restrict__ mat, uint16_t* __restrict__ rho) {
+  const float sc = (float)kBins / (hi - lo);
   const int t0 = thr[0], t1 = thr[1];
-  for (size_t i = gtid(); i < n; i += gstride()) {
-    const int b = min(max((int)((vol[i] - lo) * sc), 0), nbins - 1);
+  auto voxel = [&](float v, uint8_t& m, uint16_t& d) {
+    const int b = bin_of(v, lo, sc);
     const int c = b < t0 ? 0 : ((classes == 2 || b < t1) ? 1 : 2);
-    mat[i] = (uint8_t)cls_mat[c];
-    float r = c == 0 ? cls_rho0[0] : fminf(fmaxf(vol[i] / (0.1f * cls_murho[c]), 0.f), rho_max);
-    rho[i] = __half_as_ushort(__float2half_rn(r));
+    m = (uint8_t)(c == 0 ? cls.mat[0] : c == 1 ? cls.mat[1] : cls.mat[2]);
+    const float r = c == 0 ? cls.rho0 : fminf(fmaxf(v / (0.1f * (c == 1 ? cls.murho[1] : cls.murho[2])), 0.f), rho_max);
+    d = __half_as_ushort(__float2half_rn(r));
+  };
+  const bool wide = ((uintptr_t)vol & 15) == 0 && ((uintptr_t)mat & 3) == 0 && ((uintptr_t)rho & 7) == 0;
+  const size_t n4 = wide ? n / 4 : 0;
+  for (size_t i = gtid(); i < n4; i += gstride()) {
+    const float4 v = __ldg(reinterpret_cast<const float4*>(vol) + i);
+    uchar4 m;
+    ushort4 d;
+    voxel(v.x, m.x, d.x);
+    voxel(v.y, m.y, d.y);
+    voxel(v.z, m.z, d.z);
+    voxel(v.w, m.w, d.w);
+    reinterpret_cast<uchar4*>(mat)[i] = m;
+    reinterpret_cast<ushort4*>(rho)[i] = d;
   }
+  for (size_t i = 4 * n4 + gtid(); i < n; i += gstride()) voxel(vol[i], mat[i], rho[i]);
 }
 
 // Down-sampling by 2 per axis for the Monte Carlo step (Sec. II-C.2, II-E):
 // each 2x2x2 block becomes one voxel of the material with the block's largest
 // mass (ties to the lower id) and the density that keeps the block's summed
 // attenuation at the effective energy, sum_v murho[m_v] rho_v / (8 murho[m_b]).
-__global__ void k_bin_volume(const uint8_t* __restrict__ mat, const uint16_t* __restrict__ rho, int nx, int ny,
-                             int nz, const float* __restrict__ murho, int n_mat, uint8_t* __restrict__ mat_b,
-                             uint16_t* __restrict__ rho_b) {
+__global__ void __launch_bounds__(256) k_bin_volume(const uint8_t* __restrict__ mat, const uint16_t* __restrict__ rho,
+                                                    int nx, int ny, int nz, MaterialValues murho, int n_mat,
+                                                    uint8_t* __restrict__ mat_b, uint16_t* __restrict__ rho_b) {
   const int bx = nx / 2, by = ny / 2, bz = nz / 2;
   const size_t n = (size_t)bx * by * bz;
+  __shared__ float s_mu[kMaxMat];
+  if (threadIdx.x < kMaxMat) s_mu[threadIdx.x] = murho.v[threadIdx.x];
+  __syncthreads();
+  // a block's x neighbours as one 2- and one 4-byte word (nx is even, so rows keep the arrays' alignment)
+  const bool wide = ((uintptr_t)mat & 1) == 0 && ((uintptr_t)rho & 3) == 0;
   for (size_t i = gtid(); i < n; i += gstride()) {
-    const int x = (int)(i % bx), y = (int)((i / bx) % by), z = (int)(i / ((size_t)bx * by));
+    const size_t row = i / bx;
+    const int x = (int)(i - row * bx), y = (int)(row % by), z = (int)(row / by);
     float mass[kMaxMat];
 #pragma unroll
     for (int m = 0; m < kMaxMat; ++m) mass[m] = 0.f;
     float mu = 0.f;
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const size_t v = ((size_t)(2 * z + (q >> 2)) * ny + (2 * y + ((q >> 1) & 1))) * nx + (2 * x + (q & 1));
-      const int m = mat[v];
-      const float r = __half2float(__ushort_as_half(rho[v]));
+    for (int p = 0; p < 4; ++p) {
+      const size_t v = ((size_t)(2 * z + (p >> 1)) * ny + (2 * y + (p & 1))) * nx + 2 * x;
+      const uint32_t mm = wide ? __ldg(reinterpret_cast<const uint16_t*>(mat + v)) : mat[v] | ((uint32_t)mat[v + 1] << 8);
+      const uint32_t rr = wide ? __ldg(reinterpret_cast<const uint32_t*>(rho + v)) : rho[v] | ((uint32_t)rho[v + 1] << 16);
 #pragma unroll
-      for (int k = 0; k < kMaxMat; ++k) mass[k] += (k == m) ? r : 0.f;
-      mu = fmaf(__ldg(murho + m), r, mu);
+      for (int q = 0; q < 2; ++q) {
+        const int m = (mm >> (8 * q)) & 255u;
+        const float r = __half2float(__ushort_as_half((unsigned short)(rr >> (16 * q))));
+#pragma unroll
+        for (int k = 0; k < kMaxMat; ++k) mass[k] += (k == m) ? r : 0.f;
+        mu = fmaf(s_mu[m], r, mu);
+      }
     }
     int best = 0;
-    for (int m = 1; m < n_mat; ++m)
-      if (mass[m] > mass[best]) best = m;
+    float top = mass[0];
+#pragma unroll
+    for (int m = 1; m < kMaxMat; ++m)
+      if (m < n_mat && mass[m] > top) {
+        top = mass[m];
+        best = m;
+      }
     mat_b[i] = (uint8_t)best;
-    rho_b[i] = __half_as_ushort(__float2half_rn(mu / (8.f * __ldg(murho + best))));
+    rho_b[i] = __half_as_ushort(__float2half_rn(mu / (8.f * s_mu[best])));
   }
 }
 
@@ -356,8 +436,8 @@ __global__ void k_correct(const float* __restrict__ a, const float* __restrict__
 
 }  // namespace
 
-cudaError_t recon_bin_volume(const uint8_t* mat, const uint16_t* rho, int nx, int ny, int nz, const float* murho,
-                             int n_mat, uint8_t* mat_b, uint16_t* rho_b, cudaStream_t s) {
+cudaError_t recon_bin_volume(const uint8_t* mat, const uint16_t* rho, int nx, int ny, int nz,
+                             const MaterialValues& murho, int n_mat, uint8_t* mat_b, uint16_t* rho_b, cudaStream_t s) {
   if (nx % 2 || ny % 2 || nz % 2 || n_mat < 1 || n_mat > kMaxMat) return cudaErrorInvalidValue;
   const size_t n = (size_t)(nx / 2) * (ny / 2) * (nz / 2);
   k_bin_volume<<<blocks_for(n), 256, 0, s>>>(mat, rho, nx, ny, nz, murho, n_mat, mat_b, rho_b);
@@ -392,16 +472,23 @@ cudaError_t recon_fdk(const float* p, int n_proj, const float* d_cos, const floa
   return cudaSuccess;
 }
 
-cudaError_t recon_otsu_segment(const float* vol, size_t n, float lo, float hi, int classes, const int* d_cls_mat,
-                               const float* d_cls_murho, const float* d_cls_rho0, float rho_max, unsigned int* d_hist,
-                               int* d_thr, uint8_t* mat, uint16_t* rho, cudaStream_t s) {
-  const int nbins = 256;
-  cudaError_t e = cudaMemsetAsync(d_hist, 0, nbins * 4, s);
+size_t recon_segment_scratch() { return kBins * 4 + 16 + sizeof(OtsuScratch); }
+
+cudaError_t recon_otsu_segment(const float* vol, size_t n, float lo, float hi, int classes, const SegmentClasses& cls,
+                               float rho_max, void* scratch, unsigned int** d_hist, int** d_thr, uint8_t* mat,
+                               uint16_t* rho, cudaStream_t s) {
+  unsigned int* hist = static_cast<unsigned int*>(scratch);
+  int* thr = reinterpret_cast<int*>(hist + kBins);
+  OtsuScratch* otsu = reinterpret_cast<OtsuScratch*>(thr + 4);
+  *d_hist = hist;
+  *d_thr = thr;
+  cudaError_t e = cudaMemsetAsync(scratch, 0, recon_segment_scratch(), s);
   if (e != cudaSuccess) return e;
-  k_hist<<<blocks_for(n), 256, nbins * 4, s>>>(vol, n, lo, hi, nbins, d_hist);
-  k_otsu<<<1, 256, 0, s>>>(d_hist, nbins, classes, d_thr);
-  k_segment<<<blocks_for(n), 256, 0, s>>>(vol, n, lo, hi, nbins, d_thr, classes, d_cls_mat, d_cls_murho, d_cls_rho0,
-                                          rho_max, mat, rho);
+  // few blocks: each zeroes and sums 32 copies of the histogram
+  const int grid = blocks_for((n + 3) / 4) < 152 * 4 ? blocks_for((n + 3) / 4) : 152 * 4;
+  k_hist<<<grid, 256, 0, s>>>(vol, n, lo, hi, hist);
+  k_otsu<<<kBins - 1, kBins, 0, s>>>(hist, classes, otsu, thr);
+  k_segment<<<blocks_for((n + 3) / 4), 256, 0, s>>>(vol, n, lo, hi, thr, classes, cls, rho_max, mat, rho);
   return cudaGetLastError();
 }
 

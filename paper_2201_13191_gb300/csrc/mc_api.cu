@@ -77,6 +77,8 @@ struct mc_ctx {
   int angles_cap = 0;
   float* d_post = nullptr;  // post-processing scratch
   size_t post_cap = 0;
+  unsigned char* d_seg = nullptr;  // segmentation scratch
+  size_t seg_cap = 0;
   float* d_fdk = nullptr;  // reconstruction tables and a chunk of filtered projections
   size_t fdk_cap = 0;
   double stats[MC_STAT_N] = {};
@@ -730,6 +732,7 @@ void mc_destroy(mc_ctx* ctx) {
   cudaFree(ctx->d_angles);
   cudaFree(ctx->d_post);
   cudaFree(ctx->d_fdk);
+  cudaFree(ctx->d_seg);
   for (auto& e : ctx->ev)
     if (e) cudaEventDestroy(e);
   if (ctx->graph_exec) cudaGraphExecDestroy(ctx->graph_exec);
@@ -1311,35 +1314,34 @@ int mc_fdk(mc_ctx* ctx, const float* p, int n_proj, const float* angles, int NU,
 
 namespace {
 // Total mass attenuation (cm^2/g) of every table material at energy E (linear between nodes).
-std::vector<float> murho_at(const mc_ctx* ctx, double E) {
+MaterialValues murho_at(const mc_ctx* ctx, double E) {
   const double x = (E - ctx->E0) / ctx->dE;
   const int i = std::max(0, std::min((int)std::floor(x), ctx->n_E - 2));
   const double f = x - i;
-  std::vector<float> out(ctx->n_mat);
+  MaterialValues out = {};
   for (int m = 0; m < ctx->n_mat; ++m) {
     auto tot = [&](int j) {
       const size_t q = (size_t)m * ctx->n_E + j;
       return ctx->pe[q] + ctx->in[q] + ctx->co[q];
     };
-    out[m] = (float)(tot(i) + f * (tot(i + 1) - tot(i)));
+    out.v[m] = (float)(tot(i) + f * (tot(i + 1) - tot(i)));
   }
   return out;
 }
-}  // namespace
 
-namespace {
-// Class tables of the segmentation (Sec. II-E): the material of each class and,
-// for classes k >= 1, the mass attenuation of that material at the effective
-// energy (cm^2/g, linear between nodes); cmu[3] holds class 0's density.
-void class_tables(const mc_ctx* ctx, int classes, const int* class_material, float class_density0, float e_eff,
-                  int cm[3], float cmu[6]) {
-  const std::vector<float> mr = murho_at(ctx, e_eff);
+// Class tables of the segmentation (Sec. II-E): the material of each class,
+// the mass attenuation of that material at the effective energy (cm^2/g,
+// linear between nodes) and class 0's density.
+SegmentClasses class_tables(const mc_ctx* ctx, int classes, const int* class_material, float class_density0,
+                            float e_eff) {
+  const MaterialValues mr = murho_at(ctx, e_eff);
+  SegmentClasses c;
   for (int k = 0; k < 3; ++k) {
-    cm[k] = k < classes ? class_material[k] : 0;
-    cmu[k] = mr[cm[k]];
+    c.mat[k] = k < classes ? class_material[k] : 0;
+    c.murho[k] = mr.v[c.mat[k]];
   }
-  cmu[3] = class_density0;
-  cmu[4] = cmu[5] = 0.f;
+  c.rho0 = class_density0;
+  return c;
 }
 
 bool in_table(const mc_ctx* ctx, float E) { return E >= ctx->E0 && E <= ctx->E0 + ctx->dE * (ctx->n_E - 1); }
@@ -1373,25 +1375,15 @@ int mc_segment(mc_ctx* ctx, const float* vol, int nx, int ny, int nz, int classe
   CK(cudaSetDevice(ctx->device), "cudaSetDevice");
   (void)cudaGetLastError();
   cudaStream_t s = (cudaStream_t)stream;
-  int cm[3];
-  float cmu[6];
-  class_tables(ctx, classes, class_material, class_density0, e_eff_keV, cm, cmu);
-  // device scratch: histogram [256], thresholds [2], class materials [3], class tables [6]
-  unsigned char* d = nullptr;
-  CK(cudaMallocAsync((void**)&d, 256 * 4 + 2 * 4 + 3 * 4 + 6 * 4, s), "segmentation scratch");
-  unsigned int* hist = reinterpret_cast<unsigned int*>(d);
-  int* thr = reinterpret_cast<int*>(d + 1024);
-  int* d_cm = thr + 2;
-  float* d_cmu = reinterpret_cast<float*>(d_cm + 3);
-  cudaError_t e = cudaMemcpyAsync(d_cm, cm, sizeof(cm), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(d_cmu, cmu, sizeof(cmu), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess)
-    e = recon_otsu_segment(vol, (size_t)nx * ny * nz, mu_lo, mu_hi, classes, d_cm, d_cmu, d_cmu + 3, 30.f, hist, thr,
-                           mat_out, rho_out, s);
+  const SegmentClasses cls = class_tables(ctx, classes, class_material, class_density0, e_eff_keV);
+  CK(ensure(ctx->d_seg, ctx->seg_cap, recon_segment_scratch()), "segmentation scratch");
+  unsigned int* hist = nullptr;
+  int* thr = nullptr;
+  cudaError_t e = recon_otsu_segment(vol, (size_t)nx * ny * nz, mu_lo, mu_hi, classes, cls, 30.f, ctx->d_seg, &hist, &thr,
+                                     mat_out, rho_out, s);
   if (e == cudaSuccess && hist_out) e = cudaMemcpyAsync(hist_out, hist, 256 * 4, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess && thresholds_out) e = cudaMemcpyAsync(thresholds_out, thr, 2 * 4, cudaMemcpyDeviceToHost, s);
-  cudaFreeAsync(d, s);
-  // the host class tables must outlive their copies; the read-backs must land
+  // the read-backs must land
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "segmentation");
   return MC_OK;
@@ -1419,13 +1411,8 @@ int mc_bin_volume(mc_ctx* ctx, const uint8_t* mat, const uint16_t* rho, int nx, 
     return fail(ctx, MC_ERR_INVALID_ARG, "energy outside the table");
   CK(cudaSetDevice(ctx->device), "cudaSetDevice");
   cudaStream_t s = (cudaStream_t)stream;
-  const std::vector<float> mr = murho_at(ctx, e_eff_keV);
-  float* d = nullptr;
-  CK(cudaMallocAsync((void**)&d, mr.size() * 4, s), "bin_volume table");
-  cudaError_t e = cudaMemcpyAsync(d, mr.data(), mr.size() * 4, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = recon_bin_volume(mat, rho, nx, ny, nz, d, ctx->n_mat, mat_out, rho_out, s);
-  cudaFreeAsync(d, s);
-  // the host table must outlive the copy
+  cudaError_t e = recon_bin_volume(mat, rho, nx, ny, nz, murho_at(ctx, e_eff_keV), ctx->n_mat, mat_out, rho_out, s);
+  // the caller may release its arrays when the call returns
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "bin_volume");
   return MC_OK;
@@ -1483,29 +1470,13 @@ int mc_correct_iter(mc_ctx* ctx, const float* raw_I, const float* I0, int n_proj
   uint16_t* rho = (uint16_t*)alloc(nvox * 2);
   float* ip_sim = (float*)alloc((size_t)n_proj * simg * 4);
   float* is_sim = (float*)alloc((size_t)n_sim * simg * 4);
-  unsigned int* hist = (unsigned int*)alloc(256 * 4);
-  int* thr = (int*)alloc(2 * 4 + 3 * 4 + 6 * 4);
+  void* seg = alloc(recon_segment_scratch());
   const size_t nbin = binned ? nvox / 8 : 1;
   uint8_t* mat_b = (uint8_t*)alloc(nbin);
   uint16_t* rho_b = (uint16_t*)alloc(nbin * 2);
-  float* d_murho = (float*)alloc((size_t)ctx->n_mat * 4);
-  if (bufs.size() != 14) return release(fail(ctx, MC_ERR_OOM, "correction buffers"));
-  const std::vector<float> murho_eff = murho_at(ctx, P.e_eff_keV);
-  int* d_cls_mat = thr + 2;
-  float* d_cls_murho = reinterpret_cast<float*>(thr + 5);
-  float* d_cls_rho0 = d_cls_murho + 3;
-  {
-    int cm[3];
-    float cmu[6];
-    class_tables(ctx, P.classes, P.class_material, P.class_density0, P.e_eff_keV, cm, cmu);
-    cudaError_t e = cudaMemcpyAsync(d_cls_mat, cm, sizeof(cm), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(d_cls_murho, cmu, sizeof(cmu), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(d_murho, murho_eff.data(), murho_eff.size() * 4, cudaMemcpyHostToDevice, s);
-    // the host tables are locals: their copies must complete before they go out of scope
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return release(cuda_fail(ctx, e, "class tables"));
-  }
+  if (bufs.size() != 12) return release(fail(ctx, MC_ERR_OOM, "correction buffers"));
+  const MaterialValues murho_eff = murho_at(ctx, P.e_eff_keV);
+  const SegmentClasses cls = class_tables(ctx, P.classes, P.class_material, P.class_density0, P.e_eff_keV);
   // geometry of the simulation grid over the same panel
   const float sod = ctx->sod, sdd = ctx->sdd, pu = ctx->pu, pv = ctx->pv;
   const int nu0 = ctx->nu, nv0 = ctx->nv;
@@ -1520,8 +1491,9 @@ int mc_correct_iter(mc_ctx* ctx, const float* raw_I, const float* I0, int n_proj
     const auto t0 = std::chrono::steady_clock::now();
     int rc = mc_fdk(ctx, c, n_proj, angles, NU, NV, P.nx, P.ny, P.nz, P.dx, P.dy, P.dz, vol, stream);
     if (rc) return release(rc);
-    e = recon_otsu_segment(vol, nvox, P.mu_lo, P.mu_hi, P.classes, d_cls_mat, d_cls_murho, d_cls_rho0, 30.f, hist, thr,
-                           mat, rho, s);
+    unsigned int* hist = nullptr;
+    int* thr = nullptr;
+    e = recon_otsu_segment(vol, nvox, P.mu_lo, P.mu_hi, P.classes, cls, 30.f, seg, &hist, &thr, mat, rho, s);
     if (e != cudaSuccess) return release(cuda_fail(ctx, e, "segmentation"));
     rc = mc_load_volume(ctx, mat, rho, P.nx, P.ny, P.nz, P.dx, P.dy, P.dz, 1, stream);
     if (rc) return release(rc);
@@ -1535,7 +1507,7 @@ int mc_correct_iter(mc_ctx* ctx, const float* raw_I, const float* I0, int n_proj
     }
     if (binned) {
       // the Monte Carlo step runs on the volume down-sampled by 2 per axis (Sec. II-C.2, II-E)
-      e = recon_bin_volume(mat, rho, P.nx, P.ny, P.nz, d_murho, ctx->n_mat, mat_b, rho_b, s);
+      e = recon_bin_volume(mat, rho, P.nx, P.ny, P.nz, murho_eff, ctx->n_mat, mat_b, rho_b, s);
       if (e != cudaSuccess) return release(cuda_fail(ctx, e, "down-sampling"));
       rc = mc_load_volume(ctx, mat_b, rho_b, P.nx / 2, P.ny / 2, P.nz / 2, 2.f * P.dx, 2.f * P.dy, 2.f * P.dz, 1,
                           stream);

@@ -244,13 +244,24 @@ cudaError_t ramp_filter(const float* p, int nu, int nv, int rows, float du, floa
 cudaError_t recon_fdk(const float* p, int n_proj, const float* d_cos, const float* d_sin, int nu, int nv, float pu,
                       float pv, float sod, float sdd, int nx, int ny, int nz, float dx, float dy, float dz,
                       float* d_ramp, int chunk, float* q_tmp, float* vol, cudaStream_t s);
-cudaError_t recon_otsu_segment(const float* vol, size_t n, float lo, float hi, int classes, const int* d_cls_mat,
-                               const float* d_cls_murho, const float* d_cls_rho0, float rho_max, unsigned int* d_hist,
-                               int* d_thr, uint8_t* mat, uint16_t* rho, cudaStream_t s);
+// Segmentation: per class its material, mass attenuation at the effective energy and class 0's density; scratch: device,
+// recon_segment_scratch() bytes, where *d_hist [256] and *d_thr [2] lie afterwards.
+struct SegmentClasses {
+  int mat[3];
+  float murho[3];
+  float rho0;
+};
+size_t recon_segment_scratch();
+cudaError_t recon_otsu_segment(const float* vol, size_t n, float lo, float hi, int classes, const SegmentClasses& cls,
+                               float rho_max, void* scratch, unsigned int** d_hist, int** d_thr, uint8_t* mat,
+                               uint16_t* rho, cudaStream_t s);
 // 2x2x2 down-sampling of a segmented volume (even dims): largest-mass material, attenuation-conserving density
-// at the effective energy (murho: device [n_mat] mass attenuation there).
-cudaError_t recon_bin_volume(const uint8_t* mat, const uint16_t* rho, int nx, int ny, int nz, const float* murho,
-                             int n_mat, uint8_t* mat_b, uint16_t* rho_b, cudaStream_t s);
+// at the effective energy (murho: mass attenuation per material there).
+struct MaterialValues {
+  float v[kMaxMat];
+};
+cudaError_t recon_bin_volume(const uint8_t* mat, const uint16_t* rho, int nx, int ny, int nz,
+                             const MaterialValues& murho, int n_mat, uint8_t* mat_b, uint16_t* rho_b, cudaStream_t s);
 // c = a - ln(ip / (ip + is_scale * is)): is_scale converts the scatter image's
 // per-pixel values to the panel's pixel area when it was simulated on another grid.
 cudaError_t recon_correct(const float* a, const float* ip, const float* is, float is_scale, size_t n, float* c,
