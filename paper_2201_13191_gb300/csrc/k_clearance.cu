@@ -1,4 +1,4 @@
-// Volumes with clearance (VOX_HOP): which voxels ahead of a voxel hold the same
+// Volumes with clearance (VOX_HOP, VOX_HOP2): which voxels ahead of a voxel hold the same
 // material and density, per direction octant, so that a march takes all the
 // midpoints inside a uniform cube from one word (mc_device.cuh, Hop).
 //
@@ -6,7 +6,8 @@
 // density) pairs, at most 256) and a 3-bit code c per octant o: the cube that
 // starts at the voxel and extends r = 2^c - 1 voxels along each axis in the
 // octant's direction is uniform.  Octant bit a is set where the ray runs toward
-// smaller coordinates of axis a.
+// smaller coordinates of axis a.  A volume with more pairs keeps the codes in a
+// second word beside the voxel's own (VOX_HOP2).
 //
 // Everything is built from bit masks along x.  A cell is the 2 x 2 x 2 cube of
 // voxels at v .. v + 1; level r of a voxel says that the r^3 cells from v on
@@ -16,6 +17,8 @@
 // the seven levels serve all eight octants: about 2 words of traffic per 32
 // voxels and level instead of a distance per voxel and octant.
 #include <stdint.h>
+
+#include <algorithm>
 
 #include "mc_device.cuh"
 
@@ -32,23 +35,31 @@ __device__ __forceinline__ uint32_t voxel_key(uint32_t mat, uint32_t rho) { retu
 // every density a finite, non-negative binary16 (out->bad), the x-neighbour
 // pairs of different materials (out->changes), and a mark for every key that
 // occurs.  VEC voxels per thread and step (8: one 8-byte and one 16-byte load,
-// for arrays aligned to them).  A lane marks a key only where it differs from
-// its previous voxel's, and only if the mark is not there yet: long runs of one
-// key cost a compare.
+// for arrays aligned to them).  Marks are kept per block in shared memory and
+// merged at its end; a block that has seen more keys than a palette holds says
+// so (out->pairs) and stops marking, so that a volume with a density of its own
+// in every voxel is read at the speed of its loads (a noisy 256^3 and 128^3:
+// 160 -> 46 us together).
+constexpr int kScanWords = kKeys / 32;
 template <int VEC>
 __global__ void __launch_bounds__(256) k_scan_volume(const uint8_t* __restrict__ mat, const uint16_t* __restrict__ rho,
                                                      size_t n, uint32_t nx, int n_mat, VolumeScan* out,
                                                      uint32_t* __restrict__ seen) {
+  __shared__ uint32_t marks[kScanWords];
+  __shared__ volatile uint32_t n_keys;
+  for (int i = threadIdx.x; i < kScanWords; i += blockDim.x) marks[i] = 0u;
+  if (threadIdx.x == 0) n_keys = 0u;
+  __syncthreads();
   uint32_t last = 0xFFFFFFFFu, changes = 0;
   int bad = 0;
   auto voxel = [&](uint32_t m, uint32_t h) {
     const bool wrong = m >= (uint32_t)n_mat || h > 0x8000u || (h & 0x7C00u) == 0x7C00u;
     bad |= wrong;
     const uint32_t key = voxel_key(m, h);
-    if (wrong || key == last) return;
+    if (wrong || key == last || n_keys > (uint32_t)kMaxPalette) return;
     last = key;
     const uint32_t bit = 1u << (key & 31);
-    if (!(__ldcg(seen + (key >> 5)) & bit)) atomicOr(seen + (key >> 5), bit);
+    if (!(marks[key >> 5] & bit) && !(atomicOr(&marks[key >> 5], bit) & bit)) atomicAdd((uint32_t*)&n_keys, 1u);
   };
   const size_t stride = (size_t)gridDim.x * blockDim.x * VEC;
   for (size_t i = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * VEC; i < n; i += stride) {
@@ -85,6 +96,14 @@ __global__ void __launch_bounds__(256) k_scan_volume(const uint8_t* __restrict__
   for (int o = 16; o > 0; o >>= 1) changes += __shfl_down_sync(0xffffffffu, changes, o);
   if ((threadIdx.x & 31) == 0 && changes) atomicAdd(&out->changes, (unsigned long long)changes);
   if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(&out->bad, 1u);
+  if (n_keys > (uint32_t)kMaxPalette) {  // uniform: nothing is marked after the barrier
+    if (threadIdx.x == 0) atomicMax(&out->pairs, n_keys);
+    return;
+  }
+  for (int i = threadIdx.x; i < kScanWords; i += blockDim.x) {
+    const uint32_t w = marks[i];
+    if (w & ~__ldcg(seen + i)) atomicOr(seen + i, w);
+  }
 }
 
 // Numbers the marked keys in order (one block): pal[index] the voxel word,
@@ -93,6 +112,7 @@ __global__ void __launch_bounds__(1024) k_palette(const uint32_t* __restrict__ s
                                                   uint8_t* __restrict__ map, uint32_t* __restrict__ count) {
   __shared__ uint32_t part[1024];
   constexpr int kWords = kKeys / 32 / 1024;
+  if (*count > (uint32_t)kMaxPalette) return;  // found by the scan
   uint32_t n = 0;
   for (int k = 0; k < kWords; ++k) n += __popc(seen[threadIdx.x * kWords + k]);
   part[threadIdx.x] = n;
@@ -103,6 +123,7 @@ __global__ void __launch_bounds__(1024) k_palette(const uint32_t* __restrict__ s
     part[threadIdx.x] += v;
     __syncthreads();
   }
+  // every thread is past the test above (the barriers)
   if (threadIdx.x == 1023) *count = part[1023];
   uint32_t at = part[threadIdx.x] - n;
   for (int k = 0; k < kWords; ++k)
@@ -114,8 +135,16 @@ __global__ void __launch_bounds__(1024) k_palette(const uint32_t* __restrict__ s
     }
 }
 
-// Palette indices over the padded grid (border voxels repeat the nearest edge voxel).
-__global__ void __launch_bounds__(256) k_pack_palette(const uint8_t* __restrict__ mat, const uint16_t* __restrict__ rho,
+// What makes two voxels the same: the palette index, or the voxel word.
+template <int LAYOUT>
+__device__ __forceinline__ uint32_t entry(const uint32_t* __restrict__ vox, size_t i) {
+  return __ldg(vox + (LAYOUT == VOX_HOP2 ? 2 * i : i));
+}
+
+// Palette indices, or voxel words beside an empty word, over the padded grid (border voxels repeat the nearest edge
+// voxel).
+template <int LAYOUT>
+__global__ void __launch_bounds__(256) k_pack_clearance(const uint8_t* __restrict__ mat, const uint16_t* __restrict__ rho,
                                                       VolumeView v, const uint8_t* __restrict__ map,
                                                       uint32_t* __restrict__ out) {
   // 32-bit indices: the packed volume has fewer than 2^31 words
@@ -125,7 +154,10 @@ __global__ void __launch_bounds__(256) k_pack_palette(const uint8_t* __restrict_
     const int px = (int)(i - r * (uint32_t)v.px), pz = (int)(r / (uint32_t)v.py), py = (int)(r - pz * (uint32_t)v.py);
     const int ix = min(max(px - 1, 0), v.nx - 1), iy = min(max(py - 1, 0), v.ny - 1), iz = min(max(pz - 1, 0), v.nz - 1);
     const size_t src = ((size_t)iz * v.ny + iy) * v.nx + ix;
-    out[i] = map[voxel_key(mat[src], rho[src])];
+    if (LAYOUT == VOX_HOP2)
+      reinterpret_cast<uint2*>(out)[i] = make_uint2((uint32_t)(rho[src] & 0x7FFFu) | ((uint32_t)mat[src] << 16), 0u);
+    else
+      out[i] = map[voxel_key(mat[src], rho[src])];
   }
 }
 
@@ -135,6 +167,7 @@ __global__ void __launch_bounds__(256) k_pack_palette(const uint8_t* __restrict_
 // value (or "mixed") once and serves the cells below and above it, with the
 // x + 1 neighbours from a shuffle: 2 loads per voxel.
 constexpr int kZRun = 8;
+template <int LAYOUT>
 __global__ void __launch_bounds__(256) k_cells(const uint32_t* __restrict__ vox, int px, int py, int pz, int wpr,
                                                uint32_t* __restrict__ bits, unsigned long long* mixed) {
   const uint32_t runs = (uint32_t)((pz + kZRun - 1) / kZRun);
@@ -145,15 +178,14 @@ __global__ void __launch_bounds__(256) k_cells(const uint32_t* __restrict__ vox,
     const uint32_t t = i / (uint32_t)wpr, wi = i - t * (uint32_t)wpr;
     const int y = (int)(t % (uint32_t)py), z0 = (int)(t / (uint32_t)py) * kZRun, z1 = min(z0 + kZRun, pz);
     const int x = (int)wi * 32 + lane, xc = min(x, px - 1), xe = min(x + 1, px - 1), y1 = min(y + 1, py - 1);
-    constexpr uint32_t kMixed = 0xFFFFFFFFu;  // no palette index
+    constexpr uint32_t kMixed = 0xFFFFFFFFu;  // no palette index, no voxel word
     auto patch = [&](int z) -> uint32_t {
-      const uint32_t* r0 = vox + ((size_t)z * py + y) * px;
-      const uint32_t* r1 = vox + ((size_t)z * py + y1) * px;
-      const uint32_t a = __ldg(r0 + xc), b = __ldg(r1 + xc);
+      const size_t r0 = ((size_t)z * py + y) * px, r1 = ((size_t)z * py + y1) * px;
+      const uint32_t a = entry<LAYOUT>(vox, r0 + xc), b = entry<LAYOUT>(vox, r1 + xc);
       uint32_t an = __shfl_down_sync(0xffffffffu, a, 1), bn = __shfl_down_sync(0xffffffffu, b, 1);
       if (lane == 31) {
-        an = __ldg(r0 + xe);
-        bn = __ldg(r1 + xe);
+        an = entry<LAYOUT>(vox, r0 + xe);
+        bn = entry<LAYOUT>(vox, r1 + xe);
       }
       return a == b && a == an && a == bn ? a : kMixed;
     };
@@ -209,6 +241,7 @@ __global__ void __launch_bounds__(256) k_level(const uint32_t* __restrict__ in, 
 // of its warp reaches; the planes are turned into words in shared memory, from
 // where the warp writes row by row.
 constexpr int kCodeWarps = 4;
+template <int LAYOUT>
 __global__ void __launch_bounds__(32 * kCodeWarps) k_codes(const uint32_t* __restrict__ bits, size_t level_words, int px,
                                                            int py, int pz, int wpr, uint32_t* __restrict__ vox) {
   // [row word of the warp][bit plane, 24 used]: 16-byte rows read by all lanes at once
@@ -271,8 +304,9 @@ __global__ void __launch_bounds__(32 * kCodeWarps) k_codes(const uint32_t* __res
                   (((q.w >> lane) & 1u) << 3)) << b;
       }
       if (jx < px) {
-        uint32_t* w = vox + (size_t)jr * px + jx;
-        *w |= codes << 8;
+        const size_t at = (size_t)jr * px + jx;
+        if (LAYOUT == VOX_HOP2) vox[2 * at + 1] = codes << 8;
+        else vox[at] |= codes << 8;
       }
     }
   }
@@ -312,40 +346,51 @@ cudaError_t scan_volume(const uint8_t* mat, const uint16_t* rho, int nx, int ny,
   if (e != cudaSuccess) return e;
   auto* scan = static_cast<VolumeScan*>(scratch);
   if (((uintptr_t)mat & 7) == 0 && ((uintptr_t)rho & 15) == 0)
-    k_scan_volume<8><<<grid_of((n + 7) / 8), 256, 0, s>>>(mat, rho, n, (uint32_t)nx, n_mat, scan, scratch_seen(scratch));
+    k_scan_volume<8><<<std::min(grid_of((n + 7) / 8), 152 * 6), 256, 0, s>>>(mat, rho, n, (uint32_t)nx, n_mat, scan,
+                                                                             scratch_seen(scratch));
   else
-    k_scan_volume<1><<<grid_of(n), 256, 0, s>>>(mat, rho, n, (uint32_t)nx, n_mat, scan, scratch_seen(scratch));
+    k_scan_volume<1><<<std::min(grid_of(n), 152 * 6), 256, 0, s>>>(mat, rho, n, (uint32_t)nx, n_mat, scan,
+                                                                   scratch_seen(scratch));
   k_palette<<<1, 1024, 0, s>>>(scratch_seen(scratch), pal, scratch_map(scratch), &scan->pairs);
   e = cudaGetLastError();
   return e == cudaSuccess ? read_scan(scratch, out, s) : e;
 }
 
-cudaError_t pack_palette(const uint8_t* mat, const uint16_t* rho, int nx, int ny, int nz, void* scratch, uint32_t* vox,
-                         double* mixed, cudaStream_t s) {
+cudaError_t pack_clearance(const uint8_t* mat, const uint16_t* rho, int nx, int ny, int nz, int layout, void* scratch,
+                           uint32_t* vox, double* mixed, cudaStream_t s) {
   VolumeView v;
-  padded_dims(nx, ny, nz, VOX_HOP, &v);
+  padded_dims(nx, ny, nz, layout, &v);
   const int wpr = (v.px + 31) / 32;
   auto* scan = static_cast<VolumeScan*>(scratch);
-  k_pack_palette<<<grid_of((size_t)v.words), 256, 0, s>>>(mat, rho, v, scratch_map(scratch), vox);
-  k_cells<<<grid_of(level_words(v.px, v.py, (v.pz + kZRun - 1) / kZRun) * 32), 256, 0, s>>>(
-      vox, v.px, v.py, v.pz, wpr, scratch_levels(scratch), &scan->mixed);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = cudaMemsetAsync(&scan->mixed, 0, sizeof(scan->mixed), s);
+  if (e != cudaSuccess) return e;
+  const int g = grid_of((size_t)v.words), gc = grid_of(level_words(v.px, v.py, (v.pz + kZRun - 1) / kZRun) * 32);
+  if (layout == VOX_HOP2) {
+    k_pack_clearance<VOX_HOP2><<<g, 256, 0, s>>>(mat, rho, v, scratch_map(scratch), vox);
+    k_cells<VOX_HOP2><<<gc, 256, 0, s>>>(vox, v.px, v.py, v.pz, wpr, scratch_levels(scratch), &scan->mixed);
+  } else {
+    k_pack_clearance<VOX_HOP><<<g, 256, 0, s>>>(mat, rho, v, scratch_map(scratch), vox);
+    k_cells<VOX_HOP><<<gc, 256, 0, s>>>(vox, v.px, v.py, v.pz, wpr, scratch_levels(scratch), &scan->mixed);
+  }
+  e = cudaGetLastError();
   VolumeScan h = {};
   if (e == cudaSuccess) e = read_scan(scratch, &h, s);
   *mixed = (double)h.mixed / (double)v.words;
   return e;
 }
 
-cudaError_t build_clearance(int nx, int ny, int nz, void* scratch, uint32_t* vox, cudaStream_t s) {
+cudaError_t build_clearance(int nx, int ny, int nz, int layout, void* scratch, uint32_t* vox, cudaStream_t s) {
   VolumeView v;
-  padded_dims(nx, ny, nz, VOX_HOP, &v);
+  padded_dims(nx, ny, nz, layout, &v);
   uint32_t* bits = scratch_levels(scratch);
   const size_t lw = level_words(v.px, v.py, v.pz);
   const int wpr = (v.px + 31) / 32;
   for (int l = 0; l + 1 < kLevels; ++l)
     k_level<<<grid_of(lw), 256, 0, s>>>(bits + l * lw, (2 << l) - 1, v.py, v.pz, wpr, bits + (l + 1) * lw);
   const size_t blocks = (lw + 32 * kCodeWarps - 1) / (32 * kCodeWarps);
-  k_codes<<<(int)(blocks < 152 * 32 ? blocks : 152 * 32), 32 * kCodeWarps, 0, s>>>(bits, lw, v.px, v.py, v.pz, wpr, vox);
+  const int g = (int)(blocks < 152 * 32 ? blocks : 152 * 32);
+  if (layout == VOX_HOP2) k_codes<VOX_HOP2><<<g, 32 * kCodeWarps, 0, s>>>(bits, lw, v.px, v.py, v.pz, wpr, vox);
+  else k_codes<VOX_HOP><<<g, 32 * kCodeWarps, 0, s>>>(bits, lw, v.px, v.py, v.pz, wpr, vox);
   return cudaGetLastError();
 }
 

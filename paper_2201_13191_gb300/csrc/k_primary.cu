@@ -90,8 +90,11 @@ __global__ void __launch_bounds__(256) k_primary(const PrimaryParams P) {
     h = L / (float)n;
     VoxRay r;
     r.set(V, o, w);
-    const uint32_t w0 = __ldg(V.vox + r.voxel<LAYOUT>(V, fmaf(0.5f, h, ta)));
-    int cur = vox_mat(LAYOUT == VOX_HOP ? s_pal[w0 & 255u] : w0);
+    const int first = r.voxel<LAYOUT>(V, fmaf(0.5f, h, ta));
+    uint32_t w0, codes;
+    if constexpr (is_hop(LAYOUT)) w0 = hop_word<LAYOUT>(V, s_pal, first, codes);
+    else w0 = __ldg(V.vox + first);
+    int cur = vox_mat(w0);
     unsigned long long run = 0ull;
     auto change = [&](int m) {
       if (m == cur) return;
@@ -109,7 +112,7 @@ __global__ void __launch_bounds__(256) k_primary(const PrimaryParams P) {
       cur = m;
       run = 0ull;
     };
-    if constexpr (LAYOUT == VOX_HOP) {
+    if constexpr (is_hop(LAYOUT)) {
       // one word stands for every midpoint in its uniform cube: the same integers, count times (2048^2 panel,
       // 512^3 volume: 0.45 ms a projection against 3.6 with a gather per midpoint)
       const float3 hv = make_float3(h * r.vw.x, h * r.vw.y, h * r.vw.z);
@@ -119,9 +122,8 @@ __global__ void __launch_bounds__(256) k_primary(const PrimaryParams P) {
       for (float k = 0.f; k < nf;) {
         const float t = fmaf(k + 0.5f, h, ta);
         const float3 p = make_float3(fmaf(t, r.vw.x, r.v0.x), fmaf(t, r.vw.y, r.v0.y), fmaf(t, r.vw.z, r.v0.z));
-        const uint32_t hw = __ldg(V.vox + r.voxel_p<LAYOUT>(V, p.x, p.y, p.z));
-        const float m = fminf(hop.steps(hw, p), nf - k);
-        const uint32_t wd = s_pal[hw & 255u];
+        const uint32_t wd = hop_word<LAYOUT>(V, s_pal, r.voxel_p<LAYOUT>(V, p.x, p.y, p.z), codes);
+        const float m = fminf(hop.steps(codes, p), nf - k);
         change(vox_mat(wd));
         run += (unsigned long long)(uint32_t)m * fp16_fixed24((uint16_t)(wd & 0xffffu));
         k += m;
@@ -130,7 +132,7 @@ __global__ void __launch_bounds__(256) k_primary(const PrimaryParams P) {
     // the words of the next kAhead midpoints are loaded before any is used (the
     // step positions are known in advance, so the gathers are independent);
     // midpoints past the chord's end repeat its last one and are not summed
-    for (int k0 = 0; LAYOUT != VOX_HOP && k0 < n; k0 += kAhead) {
+    for (int k0 = 0; !is_hop(LAYOUT) && k0 < n; k0 += kAhead) {
       uint32_t wd[kAhead];
 #pragma unroll
       for (int u = 0; u < kAhead; ++u) {
@@ -184,10 +186,10 @@ cudaError_t launch_primary(const PrimaryParams& p, cudaStream_t s) {
   const int npix = p.geo.nu * p.geo.nv;
   dim3 grid((npix + block - 1) / block, p.n_angles);
   const int smem = ((p.spec.n_bins * p.tab.n_mat * 4 + 7) & ~7) + (p.shared_acc ? p.tab.n_mat * block * 8 : 0);
-  const bool brick = p.vol.layout == VOX_BRICK;
-  auto k = p.vol.layout == VOX_HOP ? (p.shared_acc ? k_primary<VOX_HOP, true> : k_primary<VOX_HOP, false>)
-           : brick                 ? (p.shared_acc ? k_primary<VOX_BRICK, true> : k_primary<VOX_BRICK, false>)
-                                   : (p.shared_acc ? k_primary<VOX_LIN, true> : k_primary<VOX_LIN, false>);
+  auto* k = p.shared_acc ? k_primary<VOX_LIN, true> : k_primary<VOX_LIN, false>;
+  if (p.vol.layout == VOX_BRICK) k = p.shared_acc ? k_primary<VOX_BRICK, true> : k_primary<VOX_BRICK, false>;
+  if (p.vol.layout == VOX_HOP) k = p.shared_acc ? k_primary<VOX_HOP, true> : k_primary<VOX_HOP, false>;
+  if (p.vol.layout == VOX_HOP2) k = p.shared_acc ? k_primary<VOX_HOP2, true> : k_primary<VOX_HOP2, false>;
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
@@ -228,7 +230,7 @@ void padded_dims(int nx, int ny, int nz, int layout, VolumeView* v) {
 size_t packed_words(int nx, int ny, int nz, int layout) {
   VolumeView v;
   padded_dims(nx, ny, nz, layout, &v);
-  return (size_t)v.words;
+  return (size_t)v.words * (layout == VOX_HOP2 ? 2 : 1);
 }
 
 cudaError_t pack_volume(const uint8_t* mat, const uint16_t* rho, int nx, int ny, int nz, int layout, uint32_t* out,

@@ -210,7 +210,7 @@ __device__ __forceinline__ float march_tau(const VolumeView& V, float3 x, float3
   r.set(V, x, w);
   const float3 hv = make_float3(h * r.vw.x, h * r.vw.y, h * r.vw.z);
   float acc = 0.f, mu = 0.f;
-  if constexpr (LAYOUT == VOX_HOP) {
+  if constexpr (is_hop(LAYOUT)) {
     // Bound by the latency of one dependent gather per uniform cube instead of the L1 data pipe's one gather per
     // step: about 21 words instead of 264 per ray of the 256^3 ellipsoids, 2e7 photons at 512^2 in 35.5 ms against
     // 69.6 on the same box; 512^3 (bricks before) 4.4 against 12.9 ms for 6 x 2e5 photons.
@@ -219,9 +219,9 @@ __device__ __forceinline__ float march_tau(const VolumeView& V, float3 x, float3
     const float nf = (float)n;
     for (float k = 0.f; k < nf;) {
       const float3 p = hop_point(r, k, h, ta, hv);
-      const uint32_t hw = __ldg(V.vox + r.voxel_p<LAYOUT>(V, p.x, p.y, p.z));
-      const float m = fminf(hop.steps(hw, p), nf - k);
-      const uint32_t wd = pal[hw & 255u];
+      uint32_t codes;
+      const uint32_t wd = hop_word<LAYOUT>(V, pal, r.voxel_p<LAYOUT>(V, p.x, p.y, p.z), codes);
+      const float m = fminf(hop.steps(codes, p), nf - k);
       acc = fmaf(m * smu[vox_mat(wd) * stride], vox_rho(wd), acc);
       k += m;
     }
@@ -268,15 +268,15 @@ __device__ __forceinline__ float2 march_tau2(const VolumeView& V, float3 x, floa
   const float3 hv = make_float3(h * r.vw.x, h * r.vw.y, h * r.vw.z);
   float acc_a = 0.f, acc_b = 0.f, mu_a = 0.f, mu_b = 0.f;
   int cur = -1;
-  if constexpr (LAYOUT == VOX_HOP) {
+  if constexpr (is_hop(LAYOUT)) {
     Hop hop;
     hop.set(r, hv, (float)n);
     const float nf = (float)n;
     for (float k = 0.f; k < nf;) {
       const float3 p = hop_point(r, k, h, ta, hv);
-      const uint32_t hw = __ldg(V.vox + r.voxel_p<LAYOUT>(V, p.x, p.y, p.z));
-      const float m = fminf(hop.steps(hw, p), nf - k);
-      const uint32_t wd = T.pal[hw & 255u];
+      uint32_t codes;
+      const uint32_t wd = hop_word<LAYOUT>(V, T.pal, r.voxel_p<LAYOUT>(V, p.x, p.y, p.z), codes);
+      const float m = fminf(hop.steps(codes, p), nf - k);
       if (vox_mat(wd) != cur) {
         cur = vox_mat(wd);
         mu_a = 0.1f * T.at(TAB_TOT, cur, ia, fa);
@@ -689,7 +689,7 @@ __device__ __forceinline__ void pseudo_particle(const TransportParams& P, const 
 // photons 13.5 / 10.4 / 9.2 ms.  The step-by-step marches keep the L1 data pipe
 // busy with 2, and the expected-value and Doppler forms spill too much beyond 2.
 constexpr int min_blocks(int layout, bool combine, bool ev, bool dop, bool hbm) {
-  return layout == VOX_HOP && !combine && !ev && !dop ? (hbm ? 4 : 3) : 2;
+  return is_hop(layout) && !combine && !ev && !dop ? (hbm ? 4 : 3) : 2;
 }
 // Flights through a linear-layout volume sum each group's optical depth
 // branch-free before looking for the interaction step (1), or test every step
@@ -1018,16 +1018,16 @@ __global__ void __launch_bounds__(256, MINB) k_transport(const TransportParams P
             return false;
           };
           int k0 = 0;
-          if constexpr (LAYOUT == VOX_HOP) {
+          if constexpr (is_hop(LAYOUT)) {
             // one word stands for the steps in its uniform cube (flight_word)
             Hop hop;
             hop.set(vr, hv, (float)n);
             const float nf = (float)n;
             for (float kn = 0.f; kn < nf && !hit;) {
               const float3 p = hop_point(vr, kn, hh, ta, hv);
-              const uint32_t hw = __ldg(V.vox + vr.voxel_p<LAYOUT>(V, p.x, p.y, p.z));
-              const float m = fminf(hop.steps(hw, p), nf - kn);
-              const uint32_t wd = T.pal[hw & 255u];
+              uint32_t codes;
+              const uint32_t wd = hop_word<LAYOUT>(V, T.pal, vr.voxel_p<LAYOUT>(V, p.x, p.y, p.z), codes);
+              const float m = fminf(hop.steps(codes, p), nf - kn);
               const float mu = my_mu[vox_mat(wd) * B] * vox_rho(wd);
               float ks;
               if (flight_word(mu, hh, tau_star, m, tau, ks)) {
@@ -1047,12 +1047,12 @@ __global__ void __launch_bounds__(256, MINB) k_transport(const TransportParams P
               consume(wd, k0, true);
             }
           }
-          for (; LAYOUT != VOX_HOP && k0 + kLook <= n && !hit; k0 += kLook) {
+          for (; !is_hop(LAYOUT) && k0 + kLook <= n && !hit; k0 += kLook) {
             uint32_t wd[kLook];
             gather_group<LAYOUT>(V, vr, k0, hh, ta, hv, wd);
             if (LAYOUT != VOX_LIN || !MC_FLIGHT_GROUP || group_reaches(wd, k0, false)) consume(wd, k0, false);
           }
-          if (LAYOUT != VOX_HOP && k0 < n && !hit) {
+          if (!is_hop(LAYOUT) && k0 < n && !hit) {
             uint32_t wd[kLook];
             gather_group<LAYOUT>(V, vr, k0, hh, ta, hv, wd);
             if (LAYOUT != VOX_LIN || !MC_FLIGHT_GROUP || group_reaches(wd, k0, true)) consume(wd, k0, true);
@@ -1317,17 +1317,27 @@ cudaError_t launch_one(const TransportParams& p, int grid, int block, int smem, 
 }
 
 // A packed volume beyond 3/4 of the 126 MB L2 streams from HBM (the line at which the layouts change, too).
-constexpr long long kL2Words = (long long)(0.75 * 126e6) / 4;
+bool beyond_l2(int layout, int words) { return (double)words * (layout == VOX_HOP2 ? 8.0 : 4.0) > 0.75 * 126e6; }
+
+template <int LAYOUT>
+cudaError_t launch_plain(const TransportParams& p, int grid, int block, int smem, cudaStream_t s) {
+  return beyond_l2(LAYOUT, p.vol.words) ? launch_one<LAYOUT, false, false, false, true>(p, grid, block, smem, s)
+                                        : launch_one<LAYOUT, false, false, false>(p, grid, block, smem, s);
+}
+template <int LAYOUT>
+void (*occupancy_kernel(bool plain, int words))(const TransportParams) {
+  if (!plain) return k_transport<LAYOUT, false, true, true, 2>;
+  return beyond_l2(LAYOUT, words) ? k_transport<LAYOUT, false, false, false, min_blocks(LAYOUT, false, false, false, true)>
+                                  : k_transport<LAYOUT, false, false, false, min_blocks(LAYOUT, false, false, false, false)>;
+}
 }  // namespace
 
 cudaError_t transport_occupancy(int block, int smem, int* blocks_per_sm, bool mesh, int layout, bool plain, int words) {
-  const bool hbm = words > kL2Words;
-  auto* k = mesh                  ? k_transport<GEO_MESH, false, false, false, 2>
-            : layout == VOX_BRICK ? k_transport<VOX_BRICK, false, false, false, 2>
-            : layout != VOX_HOP   ? k_transport<VOX_LIN, false, false, false, 2>
-            : !plain              ? k_transport<VOX_HOP, false, true, true, 2>
-            : hbm ? k_transport<VOX_HOP, false, false, false, min_blocks(VOX_HOP, false, false, false, true)>
-                  : k_transport<VOX_HOP, false, false, false, min_blocks(VOX_HOP, false, false, false, false)>;
+  void (*k)(const TransportParams) = k_transport<VOX_LIN, false, false, false, 2>;
+  if (mesh) k = k_transport<GEO_MESH, false, false, false, 2>;
+  else if (layout == VOX_BRICK) k = k_transport<VOX_BRICK, false, false, false, 2>;
+  else if (layout == VOX_HOP) k = occupancy_kernel<VOX_HOP>(plain, words);
+  else if (layout == VOX_HOP2) k = occupancy_kernel<VOX_HOP2>(plain, words);
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, block, smem);
@@ -1354,7 +1364,7 @@ cudaError_t launch_transport(const TransportParams& p, int grid, int block, cuda
   // the mesh geometry takes the global tally (the modes give the same image)
   const int variant = p.geometry == GEO_MESH
                           ? 16 | (ev ? 2 : 0) | (p.doppler ? 1 : 0)
-                          : (p.vol.layout == VOX_HOP ? 24 : p.vol.layout == VOX_BRICK ? 8 : 0) | (combine ? 4 : 0) | (ev ? 2 : 0) | (p.doppler ? 1 : 0);
+                          : (p.vol.layout == VOX_HOP2 ? 32 : p.vol.layout == VOX_HOP ? 24 : p.vol.layout == VOX_BRICK ? 8 : 0) | (combine ? 4 : 0) | (ev ? 2 : 0) | (p.doppler ? 1 : 0);
   switch (variant) {
 #define MC_LAUNCH(V, L, C, E, D) \
   case V:                        \
@@ -1380,8 +1390,7 @@ cudaError_t launch_transport(const TransportParams& p, int grid, int block, cuda
     MC_LAUNCH(18, GEO_MESH, false, true, false)
     MC_LAUNCH(19, GEO_MESH, false, true, true)
     case 24:
-      return p.vol.words > kL2Words ? launch_one<VOX_HOP, false, false, false, true>(p, grid, block, smem, s)
-                                    : launch_one<VOX_HOP, false, false, false>(p, grid, block, smem, s);
+      return launch_plain<VOX_HOP>(p, grid, block, smem, s);
     MC_LAUNCH(25, VOX_HOP, false, false, true)
     MC_LAUNCH(26, VOX_HOP, false, true, false)
     MC_LAUNCH(27, VOX_HOP, false, true, true)
@@ -1389,6 +1398,15 @@ cudaError_t launch_transport(const TransportParams& p, int grid, int block, cuda
     MC_LAUNCH(29, VOX_HOP, true, false, true)
     MC_LAUNCH(30, VOX_HOP, true, true, false)
     MC_LAUNCH(31, VOX_HOP, true, true, true)
+    case 32:
+      return launch_plain<VOX_HOP2>(p, grid, block, smem, s);
+    MC_LAUNCH(33, VOX_HOP2, false, false, true)
+    MC_LAUNCH(34, VOX_HOP2, false, true, false)
+    MC_LAUNCH(35, VOX_HOP2, false, true, true)
+    MC_LAUNCH(36, VOX_HOP2, true, false, false)
+    MC_LAUNCH(37, VOX_HOP2, true, false, true)
+    MC_LAUNCH(38, VOX_HOP2, true, true, false)
+    MC_LAUNCH(39, VOX_HOP2, true, true, true)
 #undef MC_LAUNCH
   }
   return cudaErrorInvalidValue;

@@ -52,11 +52,13 @@ struct mc_ctx {
   // volume
   bool have_volume = false;
   uint32_t* d_vox = nullptr;
+  uint32_t* d_hop = nullptr;        // words with clearance (the other layouts: d_vox)
+  size_t hop_cap = 0;
   uint32_t* d_pal = nullptr;        // palette of a volume with clearance [kMaxPalette]
   unsigned char* d_prep = nullptr;  // scratch of the volume load
   size_t pal_cap = 0, prep_cap = 0;  // packed voxel words (material | FP16 density)
   size_t vox_cap = 0;
-  int layout = VOX_LIN;
+  int layout = VOX_LIN, layout_p = VOX_LIN;  // of the transport and of the primary
   int nx = 0, ny = 0, nz = 0;
   float dx = 0, dy = 0, dz = 0;
   // spectrum
@@ -96,10 +98,24 @@ struct mc_ctx {
 
 namespace {
 
-// Share of mixed 2x2x2 cells up to which a volume gets words with clearance.  Measured by giving a growing share of
-// the object's voxels one of 16 densities: the transport takes as long as with single steps at 0.19 (64^3 cylinder),
-// 0.12 (256^3 ellipsoids) and 0.10 (512^3 ellipsoids), and the primary is faster at every share.
-constexpr double kMaxMixed = 0.10;
+// Share of mixed 2x2x2 cells up to which the transport and the primary march a volume by its clearance, by the size of
+// its plain words.  Measured with a cylinder of noise in uniform air (clearance / single steps, ms; a ray takes one word
+// per step inside the noise):
+//   share of the volume      0.07          0.20          0.38          0.57
+//   64^3,  transport      0.42 / 0.54   0.76 / 0.88   1.25 / 1.28   1.72 / 1.63   primary equal
+//   128^3, transport      0.98 / 1.39   1.87 / 2.22   3.38 / 3.26   5.02 / 4.20
+//   256^3, transport      2.18 / 2.25   4.89 / 3.86     (with two steps per voxel and ellipsoids equal at 0.18)
+//          primary        0.09 / 0.16   0.13 / 0.16   0.18 / 0.16   0.23 / 0.16
+//   512^3, transport      1.82 / 4.94   6.38 / 8.23   15.9 / 12.1
+//          primary        1.17 / 5.54   2.49 / 5.55   4.34 / 5.56   6.22 / 5.58
+struct MixedLimits {
+  double transport, primary;
+};
+MixedLimits mixed_limits(size_t bytes, size_t l2) {
+  if (bytes <= (size_t)16 << 20) return {0.30, 0.45};
+  if ((double)bytes <= 0.75 * (double)l2) return {0.12, 0.30};
+  return {0.25, 0.45};
+}
 
 // Chunk of filtered projections: 256^3 x 360 x 1024^2 takes 13.0 ms with chunks of 128 MB (each launch has its own
 // last wave of blocks), 11.8 with 512 MB.
@@ -264,10 +280,11 @@ TableView table_view(const mc_ctx* c) {
   return t;
 }
 
-VolumeView volume_view(const mc_ctx* c) {
+VolumeView volume_view(const mc_ctx* c, bool primary = false) {
   VolumeView v;
-  padded_dims(c->nx, c->ny, c->nz, c->layout, &v);
-  v.vox = c->d_vox;
+  const int layout = primary ? c->layout_p : c->layout;
+  padded_dims(c->nx, c->ny, c->nz, layout, &v);
+  v.vox = is_hop(layout) ? c->d_hop : c->d_vox;
   v.pal = c->d_pal;
   v.dx = c->dx; v.dy = c->dy; v.dz = c->dz;
   v.inv_dx = 1.f / c->dx; v.inv_dy = 1.f / c->dy; v.inv_dz = 1.f / c->dz;
@@ -449,7 +466,7 @@ int project_impl(mc_ctx* ctx, const float* angles, int n_angles, uint64_t N, uin
   int grid = 0, block = 0;
   if (primary_out) {
     pp.tab = table_view(ctx);
-    pp.vol = volume_view(ctx);
+    pp.vol = volume_view(ctx, true);
     pp.geo = geom_view(ctx);
     pp.spec = sv;
     pp.angles = ctx->d_angles;
@@ -720,6 +737,7 @@ void mc_destroy(mc_ctx* ctx) {
   cudaDeviceSynchronize();
   cudaFree(ctx->d_blob);
   cudaFree(ctx->d_vox);
+  cudaFree(ctx->d_hop);
   cudaFree(ctx->d_pal);
   cudaFree(ctx->d_prep);
   cudaFree(ctx->d_mesh_nodes);
@@ -878,43 +896,46 @@ int mc_load_volume(mc_ctx* ctx, const uint8_t* mat, const uint16_t* rho_fp16, in
     if (e != cudaSuccess) return cuda_fail(ctx, e, "volume validation");
     return fail(ctx, MC_ERR_INVALID_ARG, "volume holds an unknown material id or an invalid density");
   }
-  // Layout.  Default: words with clearance (x fastest) where the volume has few (material, density) pairs and few
-  // mixed cells, so that a march takes many midpoints from one word.  Otherwise x fastest while the packed volume
-  // fits in 3/4 of L2 (measured faster there), 4^3 bricks once it streams from HBM (every ray direction then
-  // reuses its sectors).
+  // Layout.  Default: words with clearance (x fastest) where few of the volume's cells are mixed, so that a march takes
+  // many midpoints from one word.  Otherwise x fastest while the packed volume fits in 3/4 of L2 (measured faster
+  // there), 4^3 bricks once it streams from HBM (every ray direction then reuses its sectors).  The primary gains from
+  // clearance up to a larger share of mixed cells than the transport, so a volume may be packed both ways.
+  int l2 = 0;
+  e = cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, ctx->device);
+  const size_t plain_bytes = packed_words(nx, ny, nz, VOX_LIN) * 4;
   int layout = ctx->opt.voxel_layout == 2 ? VOX_BRICK : VOX_LIN;
-  if (layout != VOX_BRICK && scan.pairs <= (uint32_t)kMaxPalette) {
-    e = ensure(ctx->d_vox, ctx->vox_cap, packed_words(nx, ny, nz, VOX_HOP));
-    // without room for the clearance scratch the volume is packed plainly
-    const size_t need = clearance_scratch_bytes(nx, ny, nz);
-    if (e == cudaSuccess && need > ctx->prep_cap) {
+  int layout_p = -1;
+  if (e == cudaSuccess && layout != VOX_BRICK) {
+    const int hop = scan.pairs <= (uint32_t)kMaxPalette ? VOX_HOP : VOX_HOP2;
+    const size_t words = packed_words(nx, ny, nz, hop), need = clearance_scratch_bytes(nx, ny, nz);
+    // without room for the larger words or the scratch the volume is packed plainly
+    bool room = words <= ctx->hop_cap || ensure(ctx->d_hop, ctx->hop_cap, words) == cudaSuccess;
+    if (room && need > ctx->prep_cap) {
       unsigned char* larger = nullptr;
-      if (cudaMalloc((void**)&larger, need) == cudaSuccess) {
+      room = cudaMalloc((void**)&larger, need) == cudaSuccess;
+      if (room) {
         // the scan's results stay
         e = cudaMemcpyAsync(larger, ctx->d_prep, scan_scratch_bytes(), cudaMemcpyDeviceToDevice, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         cudaFree(ctx->d_prep);
         ctx->d_prep = larger;
         ctx->prep_cap = need;
-      } else {
-        (void)cudaGetLastError();
       }
     }
-    if (e == cudaSuccess && need <= ctx->prep_cap) {
+    if (!room) (void)cudaGetLastError();
+    if (room && e == cudaSuccess) {
       double mixed = 1.0;
-      e = pack_palette(mat, rho_fp16, nx, ny, nz, ctx->d_prep, ctx->d_vox, &mixed, s);
-      if (e == cudaSuccess && mixed <= kMaxMixed) {
-        layout = VOX_HOP;
-        e = build_clearance(nx, ny, nz, ctx->d_prep, ctx->d_vox, s);
+      e = pack_clearance(mat, rho_fp16, nx, ny, nz, hop, ctx->d_prep, ctx->d_hop, &mixed, s);
+      const MixedLimits lim = mixed_limits(plain_bytes, (size_t)l2);
+      if (e == cudaSuccess && mixed <= lim.primary) {
+        layout_p = hop;
+        if (mixed <= lim.transport) layout = hop;
+        e = build_clearance(nx, ny, nz, hop, ctx->d_prep, ctx->d_hop, s);
       }
     }
   }
-  if (e == cudaSuccess && layout == VOX_LIN && ctx->opt.voxel_layout == 0) {
-    int l2 = 0;
-    e = cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, ctx->device);
-    if ((double)packed_words(nx, ny, nz, VOX_LIN) * 4.0 > 0.75 * (double)l2) layout = VOX_BRICK;
-  }
-  if (e == cudaSuccess && layout != VOX_HOP) {
+  if (e == cudaSuccess && !is_hop(layout)) {
+    if (ctx->opt.voxel_layout == 0 && (double)plain_bytes > 0.75 * (double)l2) layout = VOX_BRICK;
     const size_t words = packed_words(nx, ny, nz, layout);
     e = ensure(ctx->d_vox, ctx->vox_cap, words);
     if (e == cudaSuccess) e = pack_volume(mat, rho_fp16, nx, ny, nz, layout, ctx->d_vox, words, s);
@@ -924,6 +945,7 @@ int mc_load_volume(mc_ctx* ctx, const uint8_t* mat, const uint16_t* rho_fp16, in
   CK(cudaStreamSynchronize(s), "volume load");
   const size_t x_pairs = n - (size_t)ny * nz;
   ctx->layout = layout;
+  ctx->layout_p = layout_p >= 0 ? layout_p : layout;
   ctx->mat_change = x_pairs ? (double)scan.changes / (double)x_pairs : 0.0;
   ctx->nx = nx; ctx->ny = ny; ctx->nz = nz;
   ctx->dx = dx; ctx->dy = dy; ctx->dz = dz;

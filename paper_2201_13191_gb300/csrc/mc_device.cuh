@@ -241,7 +241,20 @@ struct VoxRay {
 __device__ __forceinline__ int vox_mat(uint32_t w) { return (int)((w >> 16) & 255u); }
 __device__ __forceinline__ float vox_rho(uint32_t w) { return __half2float(__ushort_as_half((unsigned short)(w & 0xffffu))); }
 
-// Steps a march may take from one word of a volume with clearance (VOX_HOP):
+// Entry idx of a volume with clearance: the voxel word, and in `codes` the word
+// with the octants (bits 8-31).
+template <int LAYOUT>
+__device__ __forceinline__ uint32_t hop_word(const VolumeView& vol, const uint32_t* pal, int idx, uint32_t& codes) {
+  if (LAYOUT == VOX_HOP2) {
+    const uint2 q = __ldg(reinterpret_cast<const uint2*>(vol.vox) + idx);
+    codes = q.y;
+    return q.x;
+  }
+  codes = __ldg(vol.vox + idx);
+  return pal[codes & 255u];
+}
+
+// Steps a march may take from one word of a volume with clearance:
 // the cube of 2^c voxels per axis that starts at step k's voxel and extends in
 // the ray's octant is uniform, so every midpoint before the ray leaves it reads
 // the same material and density.  eps (in voxels) keeps the exit inside by more

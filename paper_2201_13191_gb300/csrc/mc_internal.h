@@ -49,7 +49,9 @@ struct TableView {
 // cube and each 128-byte line a 4x4x2 slab whatever the ray direction.
 // HOP: x fastest, bits 0-7 a palette index (the words of the volume's distinct
 // (material, density) pairs), bits 8-31 the uniform cube ahead per octant (k_clearance.cu).
-enum VoxLayout { VOX_LIN = 0, VOX_BRICK = 1, VOX_HOP = 3 };
+// HOP2: the same for more pairs: 64 bits, the voxel word and then the octants (bits 8-31).
+enum VoxLayout { VOX_LIN = 0, VOX_BRICK = 1, VOX_HOP = 3, VOX_HOP2 = 4 };
+__host__ __device__ constexpr bool is_hop(int layout) { return layout == VOX_HOP || layout == VOX_HOP2; }
 // Transport geometry selector beside the voxel layouts: closed triangle-
 // mesh bodies (MeshView below) with exact flights instead of the march.
 constexpr int GEO_MESH = 2;
@@ -64,7 +66,7 @@ struct VolumeView {
   int layout;
   int nbx, nby;    // bricks along x, y (BRICK layout, padded dims)
   int px, py, pz;  // padded dims
-  int words;       // words in the packed array (last index + 1)
+  int words;       // entries of the packed array (last index + 1)
   int pxy;         // px * py
   int lin_bias;    // 0x4B000000 (1 + px + px py) mod 2^32: folds the round-down floors' offsets into the index
   int nx, ny, nz;
@@ -191,13 +193,13 @@ constexpr int kMaxPalette = 256;
 size_t scan_scratch_bytes();
 cudaError_t scan_volume(const uint8_t* mat, const uint16_t* rho, int nx, int ny, int nz, int n_mat, void* scratch,
                         uint32_t* pal, VolumeScan* out, cudaStream_t s);
-// Volumes with clearance, from a scan's scratch (of clearance_scratch_bytes) that found at most kMaxPalette
-// pairs: the palette indices into vox (padded, x fastest) and the share of 2x2x2 voxel cells that are mixed
-// (synchronises s), then the octant codes beside the indices.
+// Volumes with clearance (layout VOX_HOP from a scan that found at most kMaxPalette pairs, or VOX_HOP2), scratch of
+// clearance_scratch_bytes: pack_clearance packs the voxels into vox and measures the share of 2x2x2 voxel cells that
+// are mixed (synchronises s); build_clearance adds the octant codes.
 size_t clearance_scratch_bytes(int nx, int ny, int nz);
-cudaError_t pack_palette(const uint8_t* mat, const uint16_t* rho, int nx, int ny, int nz, void* scratch, uint32_t* vox,
-                         double* mixed, cudaStream_t s);
-cudaError_t build_clearance(int nx, int ny, int nz, void* scratch, uint32_t* vox, cudaStream_t s);
+cudaError_t pack_clearance(const uint8_t* mat, const uint16_t* rho, int nx, int ny, int nz, int layout, void* scratch,
+                           uint32_t* vox, double* mixed, cudaStream_t s);
+cudaError_t build_clearance(int nx, int ny, int nz, int layout, void* scratch, uint32_t* vox, cudaStream_t s);
 // Padded dimensions, brick counts and word count of a packed volume.
 void padded_dims(int nx, int ny, int nz, int layout, VolumeView* v);
 

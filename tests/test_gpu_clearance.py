@@ -70,6 +70,22 @@ def test_clearance_options(gpu, table_path, opt):
     assert st["nee_rays"] > 0
 
 
+@pytest.mark.parametrize("opt", [dict(), dict(nee_mode=1), dict(tally_mode=4, tile_u=8, tile_v=8)])
+@pytest.mark.parametrize("share", [0.05, 0.35])
+def test_many_pairs(gpu, table_path, share, opt):
+    """More pairs than a palette names (a core with a density of its own in every voxel): 64-bit words.  At the larger
+    share the primary alone marches by clearance."""
+    rng = np.random.default_rng(2)
+    shape = (50, 52, 46)
+    mat = np.zeros(shape, np.uint8)
+    rho = np.full(shape, 0.001205, np.float16)
+    y, x = np.meshgrid(np.linspace(-1, 1, 52), np.linspace(-1, 1, 46), indexing="ij")
+    core = np.broadcast_to(x * x + y * y < 4 * share / np.pi, shape)
+    mat[core] = MAT_WATER
+    rho[core] = rng.uniform(0.8, 1.2, core.sum()).astype(np.float16)
+    _same(gpu, _pair(gpu, table_path, mat, rho, (2.0, 1.8, 2.2), **opt), 1.1)
+
+
 @pytest.mark.parametrize("pairs", [255, 256, 257])
 def test_palette_edges(gpu, table_path, pairs):
     """The distinct (material, density) pairs around the 256 a word's palette index can name: a thin layer holds
