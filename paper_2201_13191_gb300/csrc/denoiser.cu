@@ -85,8 +85,6 @@ cudaError_t dalloc(Denoiser* d, T** p, size_t count) {
   return e;
 }
 
-size_t npix(const Denoiser* d, int n, int level) { return (size_t)n * (d->H >> level) * (d->W >> level); }
-
 // Output channels co0 .. co0 + cout of the operator whose packed weights `wts`
 // hold co_total output channels.
 cudaError_t conv(const Denoiser* d, const Layer& l, const __nv_bfloat16* x, const __nv_bfloat16* wts, const float* bias,
@@ -158,7 +156,6 @@ cudaError_t back_conv(Denoiser* d, int i, int n, const __nv_bfloat16* x, float* 
   cudaError_t e;
   Layer& l = d->L[i];
   const int lev = kLevel[i];
-  const size_t np = npix(d, n, lev);
   WgradParams wp;
   wp.x = x;
   wp.dy = d->gbuf;
@@ -169,8 +166,7 @@ cudaError_t back_conv(Denoiser* d, int i, int n, const __nv_bfloat16* x, float* 
   wp.cin = l.cin;
   wp.cout = l.cout;
   wp.err = d->err;
-  const int ktiles = (9 * l.cin + 127) / 128;
-  int splits = (int)std::max<size_t>(1, std::min<size_t>(np / 256, (size_t)(4 * 152 / ktiles + 1)));
+  const int splits = wgrad_splits(wp.n, wp.h, wp.w, wp.cin, wp.cout);
   TRY(launch_conv3x3_wgrad(wp, splits, s));
   if (gx) {
     const int c1 = split > 0 ? split : l.cin;

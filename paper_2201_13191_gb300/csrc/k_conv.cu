@@ -6,14 +6,14 @@
 //    accumulators in tensor memory; epilogue bias, optional ReLU, BF16 or FP32.
 //  - input gradient: the same kernel with the adjoint weights (flipped in space,
 //    transposed in channels: a 3x3 'same' convolution's adjoint).
-//  - weight gradient: dW[co][k] = sum_p dY[p][co] Xcol[p][k]; the tile is 128
-//    rows of k by N = C_out, the reduction over pixels runs in stages of 64
-//    pixels staged transposed into the K-major layout; CTAs split the pixels and
-//    add their FP32 partial tiles into dW.
+//  - weight gradient: both operands MN-major from tiled copies, the reduction
+//    over pixels (description at k_conv3x3_wgrad); CTAs split the pixels and add
+//    their FP32 partial tiles into dW.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "mc_internal.h"
@@ -22,28 +22,7 @@
 namespace mcx {
 namespace {
 
-constexpr int kM = 128;        // pixels (forward) or K rows (weight gradient) per CTA
-constexpr int kStageK = 64;    // reduction elements per stage
-constexpr int kKG = kStageK / 8;
 constexpr int kThreads = 128;  // four warps: one per 32 tensor-memory lanes
-
-// Weight-gradient operand tiles: the K-major no-swizzle canonical layout (core
-// matrices of 8 rows x 16 bytes) with padded strides, core matrices kLbo bytes
-// apart along K and 8-row groups kSbo apart, so that eight lanes storing the
-// same row of eight different core matrices hit eight different 16-byte bank
-// slots (the unpadded 128 / 1024-byte strides put them all on one).
-constexpr int kLbo = 128 + 16;
-constexpr int kSbo = kKG * kLbo + 16;
-template <int N>
-struct ConvSmem {
-  static constexpr int a_bytes = (kM / 8) * kSbo;
-  static constexpr int b_bytes = (N / 8) * kSbo;
-  static constexpr int stage_bytes = a_bytes + b_bytes;
-  static constexpr int bytes = 2 * stage_bytes + 1024;  // + alignment slack
-};
-__device__ __forceinline__ uint32_t wg_off(int row, int k) {
-  return (uint32_t)((row >> 3) * kSbo + (k >> 3) * kLbo + (row & 7) * 16 + (k & 7) * 2);
-}
 
 // ---------------------------------------------------------------------------
 // Forward (and input-gradient) convolution.
@@ -306,175 +285,179 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv3x3_fwd(const __grid_consta
   if (warp == 0) tc::tmem_free(tmem, ncols);
 }
 
-// Weight gradient.  CTA (blockIdx.x = k tile, blockIdx.y = pixel split).
-// Transpose of an 8 x 8 block of 16-bit values held as 8 rows of 16 bytes:
-// out[i] word m = (v[2m] element i, v[2m+1] element i).
-__device__ __forceinline__ void transpose8x8(const uint4 (&v)[8], uint4 (&o)[8]) {
-#pragma unroll
-  for (int pr = 0; pr < 4; ++pr) {
-    uint32_t lo[4], hi[4];
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      const uint32_t a = pr == 0 ? v[2 * m].x : pr == 1 ? v[2 * m].y : pr == 2 ? v[2 * m].z : v[2 * m].w;
-      const uint32_t b = pr == 0 ? v[2 * m + 1].x : pr == 1 ? v[2 * m + 1].y : pr == 2 ? v[2 * m + 1].z : v[2 * m + 1].w;
-      lo[m] = __byte_perm(a, b, 0x5410);  // element 2 pr of both rows
-      hi[m] = __byte_perm(a, b, 0x7632);  // element 2 pr + 1 of both rows
-    }
-    o[2 * pr] = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-    o[2 * pr + 1] = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-  }
-}
+// ---------------------------------------------------------------------------
+// Weight gradient dW[co][dy, dx][c] = sum_p X(y, x + dx)[c] dY(y - dy, x)[co].
+//
+// A tensor-core GEMM with the reduction over pixels p = (y, x).  Both tensors
+// are channel-minor, so both operands are MN-major.  A stage is a tile of 128
+// pixels (32 x 4, or 16 x 8 and 8 x 16 for narrow images) of X with one more
+// column on either side (rows of CC channels) and of dY with one more row above
+// and below (rows of NT channels), each fetched by one tiled copy (zero-filled
+// outside the image) in the canonical swizzled layout.  One MMA takes 16 pixels
+// (K) and all nine taps: its M rows are 128 / CC blocks of CC channels, X seen
+// from starts one pixel apart (the leading-dimension offset), i.e. dx = -1, 0, +1
+// (two MMAs at CC = 64; blocks past dx = +1 fall on rows nobody reads), and its
+// 3 NT columns are dY seen from starts one row apart, dy = +1, 0, -1.  Shared
+// memory is read once per 9 taps instead of three times with the rows' taps in
+// separate MMAs of NT columns (the 15 layers of one step: 1030 -> 690 us), and neither
+// operand passes through registers.  In the image's first and last row the MMA
+// leaves out the columns of the dy that falls outside, so that a value that is
+// not finite meets the same products as in the sum above; only where the width is
+// no multiple of 16 can one in the last column reach its dx = -1 tap too (and
+// in 8-wide tiles one in the first or last row its third dy).
+//
+// CTA (cin chunk, cout tile, split): the split's tiles, a run of neighbours (its
+// partial sums then grow, and round, like those of a run of pixels), go through a
+// ring of stages (warp 0 lane 0 copies, warp 1 lane 0 issues the MMAs); at the end
+// the four warps add the accumulators into dW (FP32 atomics).  Bound by the tensor
+// core's operand reads from shared memory and, at the deep layers, the atomics.
+// Measured over the denoiser's layers, 16 images of 256^2: 2.83 -> 0.70 ms per
+// step against threads that transposed both operands through registers.
+// ---------------------------------------------------------------------------
+constexpr int kWgPix = 128;      // pixels of a stage's tile
+constexpr int kWgXRows = 160;    // X pixels: 34 x 4, 18 x 8 or 10 x 16
+constexpr int kWgYRows = 192;    // dY pixels: 32 x 6, 16 x 10 or 8 x 18
+constexpr int kWgMaxStages = 8;
 
-// Weight gradient dW[co][k] = sum_q dY[q][co] X(q shifted by tap(k))[c(k)],
-// k = tap * C_in + c.  GEMM rows = 128 values of k (blockIdx.x), columns =
-// C_out (N), reduction over the pixels [pbeg, pend) of this CTA (blockIdx.y of
-// `splits`), 64 pixels per stage.  Both operands are K-major (pixels along K)
-// while the tensors are channel-minor, so each thread turns one 8 x 8 block
-// (8 pixels x 8 channels, eight 16-byte loads) into one core matrix (8 rows of
-// 8 pixels) by a register transpose and one 16-byte store per row.  A stage's
-// loads go out before the previous stage's MMAs are waited on (two buffers,
-// one mbarrier each); thread 0 issues the MMAs.  The partial tile is added
-// into dW (FP32 atomics).
-template <int N>
-__global__ void __launch_bounds__(kThreads) k_conv3x3_wgrad(const WgradParams p) {
+template <int CC, int NT>
+struct WgPlan {
+  static constexpr int groups = CC == 64 ? 2 : 1;  // MMAs per 16 pixels
+  static constexpr int cols = 3 * NT * groups;     // accumulator columns
+  static constexpr int ra = 2 * CC, rb = 2 * NT;   // bytes per pixel row
+  // X rows, and what the blocks past dx = +1 read after the tile's last
+  static constexpr int x_bytes = ((kWgXRows + 8) * ra + 1023) & ~1023;
+  static constexpr int dy_bytes = (kWgYRows * rb + 1023) & ~1023;
+  static constexpr int stage = x_bytes + dy_bytes;
+  // one CTA per SM where the accumulators take more than half of tensor memory
+  static constexpr int fit = ((cols > 256 ? 220 : 110) * 1024 - 1024) / stage;
+  static constexpr int stages = fit > kWgMaxStages ? kWgMaxStages : fit;
+  static constexpr int smem = stages * stage + 1024;
+};
+
+struct WgArgs {
+  float* dw;
+  int n, h, w, cin, tx, ty, tiles_x, tiles_y;  // tx x ty: the tile
+  int* err;
+};
+
+template <int CC, int NT>
+__global__ void __launch_bounds__(kThreads) k_conv3x3_wgrad(const __grid_constant__ CUtensorMap xmap,
+                                                            const __grid_constant__ CUtensorMap ymap, const WgArgs p) {
+  using P = WgPlan<CC, NT>;
   extern __shared__ unsigned char dyn_raw[];
-  unsigned char* dyn = reinterpret_cast<unsigned char*>(((uintptr_t)dyn_raw + 1023) & ~(uintptr_t)1023);
+  unsigned char* sm = reinterpret_cast<unsigned char*>(((uintptr_t)dyn_raw + 1023) & ~(uintptr_t)1023);
+  __shared__ __align__(8) uint64_t full[P::stages], empty[P::stages], done;
   __shared__ uint32_t tmem_holder;
-  __shared__ __align__(8) uint64_t mbar[2];
-  constexpr int kBUnits = (N / 8) * (kStageK / 8);          // 8 x 8 blocks of the dY operand per stage
-  constexpr int kBPer = (kBUnits + kThreads - 1) / kThreads;  // per thread
+  __shared__ volatile int abort_flag;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int K = 9 * p.cin;
-  const int krow0 = blockIdx.x * kM;
-  const long long npix = (long long)p.n * p.h * p.w;
-  const long long chunk = (npix + gridDim.y - 1) / gridDim.y;
-  const long long pbeg = (long long)blockIdx.y * chunk;
-  const long long pend = min(npix, pbeg + chunk);
-  const int n_stages = pend > pbeg ? (int)((pend - pbeg + kStageK - 1) / kStageK) : 0;
-
-  // this thread's A block: rows rg*8 .. rg*8+7 (one tap, channels c .. c+7), pixels pg*8 .. pg*8+7
-  const int rg = tid & 15, pg = tid >> 4;
-  const int k_a = krow0 + rg * 8;
-  const int tap = k_a / p.cin, c_a = k_a - tap * p.cin;
-  const int ddy = tap / 3 - 1, ddx = tap % 3 - 1;
-  const bool row_ok = k_a < K;
-
-  auto load_a = [&](int st, uint4 (&v)[8]) {
-    const long long qs = pbeg + (long long)st * kStageK + pg * 8;
-    long long t = qs / p.w;
-    int qx = (int)(qs - t * p.w);
-    int qy = (int)(t % p.h);
-    long long qn = t / p.h;
-#pragma unroll
-    for (int jj = 0; jj < 8; ++jj) {
-      v[jj] = make_uint4(0u, 0u, 0u, 0u);
-      const int yy = qy + ddy, xx = qx + ddx;
-      if (row_ok && qs + jj < pend && yy >= 0 && yy < p.h && xx >= 0 && xx < p.w)
-        v[jj] = __ldg(reinterpret_cast<const uint4*>(p.x + ((qn * p.h + yy) * p.w + xx) * p.cin + c_a));
-      if (++qx == p.w) {
-        qx = 0;
-        if (++qy == p.h) {
-          qy = 0;
-          ++qn;
-        }
-      }
-    }
-  };
-  auto load_b = [&](int st, int u, uint4 (&v)[8]) {
-    const int cg = u % (N / 8), bp = u / (N / 8);
-    const long long qs = pbeg + (long long)st * kStageK + bp * 8;
-#pragma unroll
-    for (int jj = 0; jj < 8; ++jj) {
-      v[jj] = make_uint4(0u, 0u, 0u, 0u);
-      if (qs + jj < pend && cg * 8 < p.cout)
-        v[jj] = __ldg(reinterpret_cast<const uint4*>(p.dy + (qs + jj) * p.cout + cg * 8));
-    }
-  };
-
-  if (warp == 0) tc::tmem_alloc(&tmem_holder, tmem_cols(N));
+  const int c0 = blockIdx.x * CC, n0 = blockIdx.y * NT;
+  const int per_img = p.tiles_x * p.tiles_y;
+  const long long tiles = (long long)p.n * per_img;
+  const long long first = tiles * blockIdx.z / gridDim.z;  // this CTA's tiles: a run of them
+  const int count = (int)(tiles * (blockIdx.z + 1) / gridDim.z - first);
+  const uint32_t ncols = tmem_cols(P::cols);
+  if (warp == 0) tc::tmem_alloc(&tmem_holder, ncols);
   if (tid == 0) {
-    tc::mbar_init(&mbar[0], 1);
-    tc::mbar_init(&mbar[1], 1);
+    for (int i = 0; i < P::stages; ++i) {
+      tc::mbar_init(&full[i], 1);
+      tc::mbar_init(&empty[i], 1);
+    }
+    tc::mbar_init(&done, 1);
+    abort_flag = 0;
   }
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
   const uint32_t tmem = tmem_holder;
-  bool ok = true;
-  uint4 ra[8], rb[kBPer][8];
-  if (n_stages > 0) {
-    load_a(0, ra);
-#pragma unroll
-    for (int i = 0; i < kBPer; ++i)
-      if (tid + i * kThreads < kBUnits) load_b(0, tid + i * kThreads, rb[i]);
-  }
-  for (int st = 0; st < n_stages; ++st) {
-    const int buf = st & 1;
-    unsigned char* sA = dyn + buf * ConvSmem<N>::stage_bytes;
-    unsigned char* sB = sA + ConvSmem<N>::a_bytes;
-    if (st >= 2) ok &= tc::mbar_wait(&mbar[buf], (uint32_t)((st >> 1) - 1) & 1u);
-    {
-      uint4 o[8];
-      transpose8x8(ra, o);
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-        *reinterpret_cast<uint4*>(sA + wg_off(rg * 8 + i, pg * 8)) = o[i];
-    }
-#pragma unroll
-    for (int i = 0; i < kBPer; ++i) {
-      const int u = tid + i * kThreads;
-      if (u < kBUnits) {
-        const int cg = u % (N / 8), bp = u / (N / 8);
-        uint4 o[8];
-        transpose8x8(rb[i], o);
-#pragma unroll
-        for (int r = 0; r < 8; ++r) *reinterpret_cast<uint4*>(sB + wg_off(cg * 8 + r, bp * 8)) = o[r];
-      }
-    }
-    // the next stage's loads overlap the barrier and this stage's MMAs
-    if (st + 1 < n_stages) {
-      load_a(st + 1, ra);
-#pragma unroll
-      for (int i = 0; i < kBPer; ++i)
-        if (tid + i * kThreads < kBUnits) load_b(st + 1, tid + i * kThreads, rb[i]);
-    }
-    tc::fence_async_smem();
-    __syncthreads();
-    if (tid == 0) {
-      tc::fence_after();
-      const uint32_t idesc = tc::idesc_bf16(kM, N);
-      for (int ks = 0; ks < kStageK / 16; ++ks) {
-        // k-step ks covers core-matrix columns 2 ks, 2 ks + 1
-        const uint64_t da = tc::sdesc(tc::saddr(sA) + ks * 2 * kLbo, kLbo, kSbo);
-        const uint64_t db = tc::sdesc(tc::saddr(sB) + ks * 2 * kLbo, kLbo, kSbo);
-        tc::mma_bf16(tmem, da, db, idesc, (st > 0 || ks > 0) ? 1u : 0u);
-      }
-      tc::commit(&mbar[buf]);
-    }
-  }
-  if (n_stages > 0) {
-    const int last = n_stages - 1;
-    ok &= tc::mbar_wait(&mbar[last & 1], (uint32_t)(last >> 1) & 1u);
-    if (n_stages > 1) ok &= tc::mbar_wait(&mbar[(last - 1) & 1], (uint32_t)((last - 1) >> 1) & 1u);
-  }
+  const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16);
+  for (int j = 0; j < P::cols; j += 8) tc::tmem_zero8(lane_base + (uint32_t)j);
+  tc::tmem_wait_st();
+  tc::fence_before();
+  __syncthreads();
   tc::fence_after();
-  if (!ok && tid == 0) atomicOr(p.err, 1);
-  if (ok && n_stages > 0) {
-    const int k = krow0 + warp * 32 + lane;  // this lane's accumulator row
-    const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16);
-#pragma unroll 1
-    for (int c0 = 0; c0 < N; c0 += 8) {
-      float v[8];
-      tc::tmem_ld8(lane_base + (uint32_t)c0, v);
-      if (k < K)
+
+  if (warp == 0 && lane == 0) {
+    // ---- producer
+    const uint32_t bytes = (uint32_t)((p.tx + 2) * p.ty * P::ra + p.tx * (p.ty + 2) * P::rb);
+    int issued = 0;
+    for (int st = 0; st < count; ++st) {
+      const int slot = st % P::stages;
+      if (st >= P::stages && !tc::mbar_wait(&empty[slot], (uint32_t)((st / P::stages) - 1) & 1u)) {
+        abort_flag = 1;
+        break;
+      }
+      if (abort_flag) break;
+      const long long t = first + st;
+      const int img = (int)(t / per_img), r = (int)(t - (long long)img * per_img);
+      const int y0 = (r / p.tiles_x) * p.ty, x0 = (r % p.tiles_x) * p.tx;
+      unsigned char* xs = sm + slot * P::stage;
+      tc::mbar_expect_tx(&full[slot], bytes);
+      tc::tma_load_4d(xs, &xmap, &full[slot], c0, x0 - 1, y0, img);
+      tc::tma_load_4d(xs + P::x_bytes, &ymap, &full[slot], n0, x0, y0 - 1, img);
+      ++issued;
+    }
+    if (abort_flag)  // let the copies still in flight land before the CTA can exit
+      for (int st = max(0, issued - P::stages); st < issued; ++st)
+        tc::mbar_wait(&full[st % P::stages], (uint32_t)(st / P::stages) & 1u);
+  } else if (warp == 1 && lane == 0) {
+    // ---- MMA issuer; operands MN-major (instruction descriptor bits 15 and 16)
+    constexpr uint32_t mn = (1u << 15) | (1u << 16);
+    // the MMA's second 8 pixels of X: the next ones, or the next row's of an 8-wide tile
+    const uint32_t next8 = (uint32_t)((p.tx == 8 ? 10 : 8) * P::ra), pitch = (uint32_t)(p.tx * P::rb);
+    for (int st = 0; st < count; ++st) {
+      const int slot = st % P::stages;
+      if (!tc::mbar_wait(&full[slot], (uint32_t)(st / P::stages) & 1u)) {
+        abort_flag = 1;
+        break;
+      }
+      tc::fence_after();
+      const int r = (int)((first + st) % per_img);
+      const int y0 = (r / p.tiles_x) * p.ty, wx = p.w - (r % p.tiles_x) * p.tx;
+      const uint32_t xa = tc::saddr(sm + slot * P::stage), ya = xa + P::x_bytes;
+      for (int i = 0; i < kWgPix / 16; ++i) {
+        const int ky = (i * 16) / p.tx, kx = (i * 16) % p.tx, y = y0 + ky;
+        if (y >= p.h || kx >= wx) continue;  // outside the image
+        // column blocks j = 0, 1, 2 read dY at row y - 1 + j (an 8-wide tile's MMA has row y + 1 as well)
+        const int j0 = y == 0 && p.tx != 8 ? 1 : 0, j1 = y == p.h - 1 ? 2 : 3;
+        const uint32_t idesc = tc::idesc_bf16(128, (j1 - j0) * NT) | mn;
+        const uint64_t db = tc::sdesc_mn(ya + (uint32_t)(i * 16 * P::rb) + (uint32_t)j0 * pitch, pitch, 8u * P::rb, P::rb);
 #pragma unroll
-        for (int j = 0; j < 8; ++j)
-          if (c0 + j < p.cout) atomicAdd(p.dw + (long long)(c0 + j) * K + k, v[j]);
+        for (int g = 0; g < P::groups; ++g) {
+          // 128 / CC blocks one pixel apart, from dx = -1 (or +1, the second group) on
+          const uint64_t da = tc::sdesc_mn(xa + (uint32_t)((ky * (p.tx + 2) + kx + 2 * g) * P::ra), P::ra, next8, P::ra);
+          tc::mma_bf16(tmem + (uint32_t)((g * 3 + j0) * NT), da, db, idesc, 1u);
+        }
+      }
+      tc::commit(&empty[slot]);
+    }
+    tc::commit(&done);
+  }
+  __syncwarp();
+  bool ok = tc::mbar_wait(&done, 0);
+  tc::fence_after();
+  ok = __syncthreads_and(ok && !abort_flag) != 0;
+  if (!ok && tid == 0) atomicOr(p.err, 1);
+  if (ok && count > 0) {
+    // accumulator row = block of CC channels (dx) x channel
+    const int m = warp * 32 + lane, c = m % CC, blk = m / CC;
+#pragma unroll 1
+    for (int a = 0; a < 3 * P::groups; ++a) {
+      const int dy = 2 - a % 3, dx = blk + 2 * (a / 3);
+      const bool use = dx < 3;
+      float* dst = p.dw + (size_t)n0 * 9 * p.cin + (size_t)(3 * dy + dx) * p.cin + c0 + c;
+#pragma unroll 1
+      for (int j0 = 0; j0 < NT; j0 += 8) {
+        float v[8];
+        tc::tmem_ld8(lane_base + (uint32_t)(a * NT + j0), v);
+        if (use)
+#pragma unroll
+          for (int j = 0; j < 8; ++j) atomicAdd(dst + (size_t)(j0 + j) * 9 * p.cin, v[j]);
+      }
     }
   }
   tc::fence_before();
   __syncthreads();
-  if (warp == 0) tc::tmem_free(tmem, tmem_cols(N));
+  if (warp == 0) tc::tmem_free(tmem, ncols);
 }
 
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no link
@@ -645,14 +628,54 @@ cudaError_t launch_fwd_n(const ConvParams& p, cudaStream_t s) {
     return launch_fwd_kernel<N, false>(map, a, gx, gy, smem, s);
 }
 
-template <int N>
+CUtensorMapSwizzle swizzle_of(int row_bytes) {
+  return row_bytes == 128 ? CU_TENSOR_MAP_SWIZZLE_128B
+                          : row_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B;
+}
+
+// Map of an NHWC BF16 tensor with boxes of `ch` channels x bw x bh pixels of one image.
+bool nhwc_map(EncodeTiledFn enc, CUtensorMap* map, const void* x, int n, int h, int w, int c, int ch, int bw, int bh) {
+  const cuuint64_t dims[4] = {(cuuint64_t)c, (cuuint64_t)w, (cuuint64_t)h, (cuuint64_t)n};
+  const cuuint64_t strides[3] = {(cuuint64_t)c * 2, (cuuint64_t)c * 2 * w, (cuuint64_t)c * 2 * w * h};
+  const cuuint32_t box[4] = {(cuuint32_t)ch, (cuuint32_t)bw, (cuuint32_t)bh, 1u};
+  const cuuint32_t estr[4] = {1u, 1u, 1u, 1u};
+  return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void*)x, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+             swizzle_of(2 * ch), CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+int wgrad_tile(int w) { return w > 16 ? 32 : w > 8 ? 16 : 8; }
+
+template <int CC, int NT>
 cudaError_t launch_wgrad_n(const WgradParams& p, int splits, cudaStream_t s) {
-  const int smem = ConvSmem<N>::bytes;
-  cudaError_t e = cudaFuncSetAttribute(k_conv3x3_wgrad<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  using P = WgPlan<CC, NT>;
+  EncodeTiledFn enc = encode_tiled();
+  if (!enc) return cudaErrorNotSupported;
+  WgArgs a;
+  a.tx = wgrad_tile(p.w);
+  a.ty = kWgPix / a.tx;
+  CUtensorMap xmap, ymap;
+  if (!nhwc_map(enc, &xmap, p.x, p.n, p.h, p.w, p.cin, CC, a.tx + 2, a.ty) ||
+      !nhwc_map(enc, &ymap, p.dy, p.n, p.h, p.w, p.cout, NT, a.tx, a.ty + 2))
+    return cudaErrorInvalidValue;
+  cudaError_t e = cudaFuncSetAttribute(k_conv3x3_wgrad<CC, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, P::smem);
   if (e != cudaSuccess) return e;
-  const int ktiles = (9 * p.cin + kM - 1) / kM;
-  k_conv3x3_wgrad<N><<<dim3(ktiles, splits), kThreads, smem, s>>>(p);
+  a.dw = p.dw;
+  a.n = p.n;
+  a.h = p.h;
+  a.w = p.w;
+  a.cin = p.cin;
+  a.tiles_x = (p.w + a.tx - 1) / a.tx;
+  a.tiles_y = (p.h + a.ty - 1) / a.ty;
+  a.err = p.err;
+  k_conv3x3_wgrad<CC, NT><<<dim3(p.cin / CC, p.cout / NT, splits), kThreads, P::smem, s>>>(xmap, ymap, a);
   return cudaGetLastError();
+}
+
+template <int CC>
+cudaError_t launch_wgrad_c(const WgradParams& p, int splits, cudaStream_t s) {
+  if (p.cout % 64 == 0) return launch_wgrad_n<CC, 64>(p, splits, s);
+  if (p.cout % 32 == 0) return launch_wgrad_n<CC, 32>(p, splits, s);
+  return launch_wgrad_n<CC, 16>(p, splits, s);
 }
 
 }  // namespace
@@ -687,13 +710,31 @@ cudaError_t launch_conv3x3_fwd(const ConvParams& p, cudaStream_t s) {
   }
 }
 
+// Channel chunks of 64, 32 or 16 (whichever divides the count); x and dy 16-byte aligned.
 cudaError_t launch_conv3x3_wgrad(const WgradParams& p, int splits, cudaStream_t s) {
-  if (p.cin % 16 || p.cout % 16 || p.cout > 256 || p.cin < 16 || splits < 1) return cudaErrorInvalidValue;
-  if (p.cout <= 16) return launch_wgrad_n<16>(p, splits, s);
-  if (p.cout <= 32) return launch_wgrad_n<32>(p, splits, s);
-  if (p.cout <= 64) return launch_wgrad_n<64>(p, splits, s);
-  if (p.cout <= 128) return launch_wgrad_n<128>(p, splits, s);
-  return launch_wgrad_n<256>(p, splits, s);
+  if (p.cin % 16 || p.cout % 16 || p.cout > 256 || p.cin < 16 || p.cout < 16 || splits < 1 || splits > 65535 ||
+      ((uintptr_t)p.x & 15) || ((uintptr_t)p.dy & 15))
+    return cudaErrorInvalidValue;
+  if (p.cin % 64 == 0) return launch_wgrad_c<64>(p, splits, s);
+  if (p.cin % 32 == 0) return launch_wgrad_c<32>(p, splits, s);
+  return launch_wgrad_c<16>(p, splits, s);
+}
+
+// CTAs that share the pixels: 608 per 128 rows of (tap, channel), each with 256
+// pixels at least, rounded up to whole waves (one CTA per SM where its
+// accumulators take more than half of tensor memory, else two).  The first sets
+// the length of an FP32 sum and so its error, which grows with it (32 -> 32
+// channels at 16 x 256^2 against FP64: 7.6e-6, 3.7e-6 and 1.8e-6 of the norm with
+// 152, 304 and 608 CTAs).  Whole waves: 32 -> 32, 203 CTAs 48 us, 304 37; 64 -> 64
+// at 128^2, 122 CTAs 40 us, 152 32; 128 -> 128 at 64^2, 272 CTAs 42 us, 304 40.
+int wgrad_splits(int n, int h, int w, int cin, int cout) {
+  const int cc = cin % 64 == 0 ? 64 : cin % 32 == 0 ? 32 : 16, nt = cout % 64 == 0 ? 64 : cout % 32 == 0 ? 32 : 16;
+  const int tx = wgrad_tile(w), ty = kWgPix / tx, ktiles = (9 * cin + 127) / 128;
+  const long long np = (long long)n * h * w, tiles = (long long)n * ((h + ty - 1) / ty) * ((w + tx - 1) / tx);
+  const int ctas = (cin / cc) * (cout / nt), wave = 3 * nt * (cc == 64 ? 2 : 1) > 256 ? 152 : 304;
+  const long long least = std::max(1ll, std::min(np / 256, (608ll + ktiles - 1) / ktiles));
+  const long long splits = (least * ctas + wave - 1) / wave * wave / ctas;
+  return (int)std::min(std::max(splits, least), tiles);
 }
 
 }  // namespace mcx

@@ -232,6 +232,7 @@ struct WgradParams {
 };
 cudaError_t launch_conv3x3_fwd(const ConvParams& p, cudaStream_t s);
 cudaError_t launch_conv3x3_wgrad(const WgradParams& p, int splits, cudaStream_t s);
+int wgrad_splits(int n, int h, int w, int cin, int cout);
 
 // Correction plumbing (k_recon.cu)
 cudaError_t recon_log_norm(const float* I, const float* I0, size_t img, size_t n, float* a, cudaStream_t s);

@@ -33,6 +33,16 @@ __device__ __forceinline__ uint64_t sdesc_swz(uint32_t addr, uint32_t sbo, int r
          ((uint64_t)1 << 46) | (layout << 61);
 }
 
+// Descriptor of an MN-major operand in a swizzled canonical layout: K rows of
+// `row_bytes` (32, 64 or 128: that many bytes of consecutive M or N elements),
+// 8-row groups `sbo` bytes apart along K, the next row_bytes / 2 elements along M
+// or N `lbo` bytes away.
+__device__ __forceinline__ uint64_t sdesc_mn(uint32_t addr, uint32_t lbo, uint32_t sbo, int row_bytes) {
+  const uint64_t layout = row_bytes == 128 ? 2ull : (row_bytes == 64 ? 4ull : 6ull);
+  return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)((lbo >> 4) & 0x3FFF) << 16) |
+         ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | ((uint64_t)1 << 46) | (layout << 61);
+}
+
 // Instruction descriptor of kind::f16: FP32 accumulator, BF16 A and B, both
 // K-major, M x N tile.
 __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
@@ -117,11 +127,11 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
   for (int j = 0; j < 8; ++j) v[j] = __uint_as_float(r[j]);
 }
 
-// Byte offset of element (row, k) in a K-major canonical tile whose K extent
-// is kgroups x 8: [row/8][k/8][row%8][k%8] (lbo = 128, sbo = kgroups * 128).
-__device__ __forceinline__ uint32_t canon_off(int row, int k, int kgroups) {
-  return (uint32_t)((((row >> 3) * kgroups + (k >> 3)) * 8 + (row & 7)) * 16 + (k & 7) * 2);
+// Zeros to 8 consecutive columns of this thread's tensor-memory lane (tmem_wait_st before they are used).
+__device__ __forceinline__ void tmem_zero8(uint32_t taddr) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1};" ::"r"(taddr), "r"(0) : "memory");
 }
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 }  // namespace tc
 }  // namespace mcx
