@@ -431,8 +431,9 @@ def _event_time(torch, stream, fn, reps=5, warm=2):
 
 
 def packed_words(shape, voxel_layout, props):
-    """Words of the library's packed volume: a one-voxel border, x fastest, or
-    4x4x4 bricks (the default switches to bricks beyond 3/4 of L2)."""
+    """Words of the library's plain packed volume: a one-voxel border, x fastest,
+    or 4x4x4 bricks (by default beyond 3/4 of L2).  Clearance words, the usual
+    packing, have as many words as the first, of 4 or 8 bytes."""
     nz, ny, nx = shape
     px, py, pz = nx + 2, ny + 2, nz + 2
     lin = px * py * pz
@@ -446,7 +447,9 @@ def packed_words(shape, voxel_layout, props):
 def memory_roofline(torch, props, shape, layout_words, steps_per_s, stream):
     """Voxel-gather roofline of the transport at the memory level the packed
     volume lives in.  Algorithmic bytes: 3 per march step (1-byte material +
-    2-byte FP16 density); the kernel reads them as one 4-byte word.  Peak:
+    2-byte FP16 density).  Over plain words the kernel reads a 4-byte word per
+    step; over clearance words one per uniform cube of voxels, so that the
+    fraction counts bytes of steps it did not have to read.  Peak:
     coalesced streaming reads (mc_probe_stream) over a buffer the size of the
     packed volume, measured live: from L2 when the buffer fits, from HBM when
     it does not.  Secondary figure: random 4-byte gathers (mc_probe_gather)

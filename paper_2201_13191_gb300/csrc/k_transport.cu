@@ -213,7 +213,8 @@ __device__ __forceinline__ float march_tau(const VolumeView& V, float3 x, float3
   if constexpr (is_hop(LAYOUT)) {
     // Bound by the latency of one dependent gather per uniform cube instead of the L1 data pipe's one gather per
     // step: about 21 words instead of 264 per ray of the 256^3 ellipsoids, 2e7 photons at 512^2 in 35.5 ms against
-    // 69.6 on the same box; 512^3 (bricks before) 4.4 against 12.9 ms for 6 x 2e5 photons.
+    // 69.6 on the same box (28.8 since, with histories from a common counter, three blocks per SM and closed-form
+    // flights); 512^3 (bricks before) 4.4 against 12.9 ms for 6 x 2e5 photons.
     Hop hop;
     hop.set(r, hv, (float)n);
     const float nf = (float)n;
