@@ -188,32 +188,195 @@ __global__ void __launch_bounds__(Plan<LOGN>::threads) k_ramp_spectrum(const flo
   middle<LOGN>(sh, t, tw, nullptr, out);
 }
 
-// Filters rows 2 b and 2 b + 1 (b the transform's number).  A row holding a
-// value that is not finite (or close to overflow) would spoil the other one:
-// it enters as zeros and its outputs are summed directly.
+// The weighted value of pixel i of a row at height v, as the direct sum takes it.
+__device__ __forceinline__ float weighted(float x, float v, int i, int nu, float du, float sod) {
+  const float u = ((float)i - 0.5f * (float)(nu - 1)) * du;
+  return x * sod * rsqrtf(sod * sod + u * u + v * v);
+}
+
+// A transform rounds every output to the size of its largest difference; a direct sum rounds each term to its own.  The
+// two agree (a few units of 2^-24 of the row's values) while no difference stands out.  Differences above
+// 3 mean|x| + 6 mean|d| are therefore left out of the transform and added with their taps G(i - j), and pixels above
+// kPixel times mean|x| (or not finite) with the taps h(i - j), whose zeros and 1 / n^2 keep such a pixel in its place.
+// There can be few of either (their share of the sums), and a row of noise, or of an object that fills a sixth of it, has
+// none.  Rows whose sums differ in their binary exponent are brought to one size (powers of two), since the two rows of a
+// transform share its rounding.
+constexpr float kPixel = 16.f;
+constexpr float kHuge = 1e30f;
+
+template <int LOGN>
+struct Large {
+  static constexpr int words = Plan<LOGN>::N / 64 + 1;  // nu + 1 bits
+  uint32_t pixel[2][words], step[2][words];             // of the transform's two rows
+};
+
+// Of a transform's two rows: sum of |x|, sum and largest of |d| (its bits: above infinity's where it is no number).
+struct RowSize {
+  float2 x, d;
+  uint32_t ma, mb;
+  __device__ __forceinline__ void add(float2 dd) {
+    d.x += fabsf(dd.x);
+    d.y += fabsf(dd.y);
+    ma = max(ma, __float_as_uint(dd.x) & 0x7FFFFFFFu);
+    mb = max(mb, __float_as_uint(dd.y) & 0x7FFFFFFFu);
+  }
+  // Largest ordinary difference; the rows of few pixels have few to take a mean of.
+  __device__ __forceinline__ float2 limit(int nu) const {
+    const float n = 3.f / (float)nu, m = 6.f / (float)(nu + 64);
+    return make_float2(fmaf(n, x.x, m * d.x), fmaf(n, x.y, m * d.y));
+  }
+};
+
+// Over a transform's threads; a barrier of the block lies between what its threads wrote before and what they read
+// afterwards.
+template <int LOGN>
+__device__ __forceinline__ RowSize row_size(RowSize s, RowSize* part, int t) {
+  constexpr int T = Plan<LOGN>::T, seg = T < 32 ? T : 32;
+#pragma unroll
+  for (int o = seg / 2; o > 0; o >>= 1) {
+    s.x.x += __shfl_xor_sync(0xffffffffu, s.x.x, o);
+    s.x.y += __shfl_xor_sync(0xffffffffu, s.x.y, o);
+    s.d.x += __shfl_xor_sync(0xffffffffu, s.d.x, o);
+    s.d.y += __shfl_xor_sync(0xffffffffu, s.d.y, o);
+  }
+  const uint32_t lanes = seg == 32 ? 0xffffffffu : 0xffffu << (threadIdx.x & 16);
+  s.ma = __reduce_max_sync(lanes, s.ma);
+  s.mb = __reduce_max_sync(lanes, s.mb);
+  if (t % seg == 0) part[t / seg] = s;
+  __syncthreads();
+  s = part[0];
+#pragma unroll
+  for (int i = 1; i < T / seg; ++i) {
+    s.x = cadd(s.x, part[i].x);
+    s.d = cadd(s.d, part[i].d);
+    s.ma = max(s.ma, part[i].ma);
+    s.mb = max(s.mb, part[i].mb);
+  }
+  return s;
+}
+
+// Marks the large pixels and differences of the rows in sh (weighted values, whose sums of |x| are `sum`) and leaves the
+// differences without them there, each thread its own places; returns the sums of |x| without the large pixels.  All
+// threads of the block call it.
+template <int LOGN>
+__device__ __noinline__ float2 take_large(float2* sh, Large<LOGN>* large, RowSize* part, float2 sum, int nu, int t) {
+  constexpr int T = Plan<LOGN>::T, words = Large<LOGN>::words;
+  uint32_t* const mark = &large->pixel[0][0];
+  for (int i = t; i < 4 * words; i += T) mark[i] = 0u;
+  __syncthreads();
+  const float n = (float)nu;
+  for (;;) {  // every round but the last takes a pixel at least
+    const float la = sum.x < kHuge ? kPixel * sum.x : 0.1f * kHuge * n, lb = sum.y < kHuge ? kPixel * sum.y : 0.1f * kHuge * n;
+    bool took = false;
+    RowSize s = {};
+#pragma unroll 1
+    for (int k = 0; k < 16; ++k) {
+      const int i = t + k * T;
+      float2 x = sh[padded(i)];
+      if (!(fabsf(x.x) * n <= la)) {
+        atomicOr(&large->pixel[0][i >> 5], 1u << (i & 31));
+        x.x = 0.f;
+        took = true;
+      }
+      if (!(fabsf(x.y) * n <= lb)) {
+        atomicOr(&large->pixel[1][i >> 5], 1u << (i & 31));
+        x.y = 0.f;
+        took = true;
+      }
+      sh[padded(i)] = x;
+      s.x = cadd(s.x, make_float2(fabsf(x.x), fabsf(x.y)));
+    }
+    took = __syncthreads_or(took);
+    sum = row_size<LOGN>(s, part, t).x;
+    if (!took) break;
+  }
+  float2 d[16];
+  RowSize s = {};
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    const int i = t + k * T;
+    d[k] = sh[padded(i)];
+    if (i > 0) d[k] = csub(d[k], sh[padded(i - 1)]);
+    s.add(d[k]);
+  }
+  __syncthreads();
+  s = row_size<LOGN>(s, part, t);
+  s.x = sum;
+  const float2 lim = s.limit(nu);
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    const int i = t + k * T;
+    if (fabsf(d[k].x) > lim.x) {
+      atomicOr(&large->step[0][i >> 5], 1u << (i & 31));
+      d[k].x = 0.f;
+    }
+    if (fabsf(d[k].y) > lim.y) {
+      atomicOr(&large->step[1][i >> 5], 1u << (i & 31));
+      d[k].y = 0.f;
+    }
+    sh[padded(i)] = d[k];
+  }
+  return sum;
+}
+
+// Adds what the large pixels and differences of a row (p, at height v) contribute to the outputs that this thread stored
+// in q; gs: G, see ramp_kernel.
+template <int LOGN>
+__device__ __noinline__ void add_large(const float* __restrict__ p, float* __restrict__ q, const uint32_t* pixel,
+                                       const uint32_t* step, const float* __restrict__ gs, int nu, float du, float v,
+                                       float sod, int t) {
+  using P = Plan<LOGN>;
+  uint32_t any = 0u;
+  for (int k = 0; k < Large<LOGN>::words; ++k) any |= pixel[k] | step[k];
+  if (!any) return;
+  const float h0 = 0.25f / (du * du), c = 1.f / (9.8696044f * du * du);
+  float acc[16] = {};
+  for (int b = 0; b < Large<LOGN>::words; ++b) {
+    for (uint32_t m = pixel[b]; m; m &= m - 1) {
+      const int j = 32 * b + __ffs(m) - 1;
+      const float x = weighted(__ldg(p + j), v, j, nu, du, sod);
+#pragma unroll
+      for (int k = 0; k < 16; ++k) {
+        const int d = t + k * P::T - j;
+        acc[k] = fmaf(x, d == 0 ? h0 : ((d & 1) ? -c / ((float)d * (float)d) : 0.f), acc[k]);
+      }
+    }
+    for (uint32_t m = step[b]; m; m &= m - 1) {
+      const int j = 32 * b + __ffs(m) - 1;
+      auto at = [&](int i) -> float {  // the row without its large pixels
+        return i < 0 || i >= nu || ((pixel[i >> 5] >> (i & 31)) & 1u) ? 0.f : weighted(__ldg(p + i), v, i, nu, du, sod);
+      };
+      const float x = at(j) - at(j - 1);
+#pragma unroll
+      for (int k = 0; k < 16; ++k) acc[k] = fmaf(x, __ldg(gs + ((t + k * P::T - j) & (P::N - 1))), acc[k]);
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    const int i = t + k * P::T;
+    if (i < nu) q[i] = fmaf(acc[k], du, q[i]);
+  }
+}
+
+// Filters rows 2 b and 2 b + 1 (b the transform's number); ramp, tw, g: see launch.
 template <int LOGN>
 __global__ void __launch_bounds__(Plan<LOGN>::threads) k_ramp_filter(const float* __restrict__ p, int nu, int nv,
                                                                      int rows, float du, float dv, float sod,
+                                                                     const float* __restrict__ ramp,
                                                                      const float2* __restrict__ tw,
                                                                      const float2* __restrict__ g,
                                                                      float* __restrict__ q) {
   using P = Plan<LOGN>;
   extern __shared__ float2 sh_all[];
-  __shared__ int bad[2 * P::per_block];
+  __shared__ RowSize part[P::per_block][P::T < 32 ? 1 : P::T / 32];
+  __shared__ Large<LOGN> large[P::per_block];
   const int f = threadIdx.x / P::T, t = threadIdx.x % P::T;
   float2* sh = sh_all + f * P::slot;
   const int r0 = 2 * (blockIdx.x * P::per_block + f);
-  if (threadIdx.x < 2 * P::per_block) bad[threadIdx.x] = 0;
-  __syncthreads();
   const float va = ((float)(r0 % nv) - 0.5f * (float)(nv - 1)) * dv;
   const float vb = ((float)((r0 + 1) % nv) - 0.5f * (float)(nv - 1)) * dv;
   const float* pa = p + (size_t)r0 * nu;
   const bool has_b = r0 + 1 < rows;
-  // the weighted value, as the direct sum takes it
-  auto weighted = [&](float x, float vv, int i) -> float {
-    const float uu = ((float)i - 0.5f * (float)(nu - 1)) * du;
-    return x * sod * rsqrtf(sod * sod + uu * uu + vv * vv);
-  };
   float2 v[16];
   if (r0 < rows) {
 #pragma unroll
@@ -222,28 +385,38 @@ __global__ void __launch_bounds__(Plan<LOGN>::threads) k_ramp_filter(const float
       v[k] = make_float2(i < nu ? __ldg(pa + i) : 0.f, i < nu && has_b ? __ldg(pa + nu + i) : 0.f);
     }
   }
-  bool bad_a = false, bad_b = false;
+  RowSize size = {};
 #pragma unroll
   for (int k = 0; k < 16; ++k) {
     const int i = t + k * P::T;
-    v[k] = r0 < rows && i < nu ? make_float2(weighted(v[k].x, va, i), weighted(v[k].y, vb, i)) : make_float2(0.f, 0.f);
-    bad_a |= !(fabsf(v[k].x) < 1e30f);
-    bad_b |= !(fabsf(v[k].y) < 1e30f);
+    v[k] = r0 < rows && i < nu ? make_float2(weighted(v[k].x, va, i, nu, du, sod), weighted(v[k].y, vb, i, nu, du, sod))
+                               : make_float2(0.f, 0.f);
+    size.x = cadd(size.x, make_float2(fabsf(v[k].x), fabsf(v[k].y)));
     sh[padded(i)] = v[k];
   }
-  if (bad_a) bad[2 * f] = 1;
-  if (bad_b) bad[2 * f + 1] = 1;
   __syncthreads();
-  bad_a = bad[2 * f] != 0;
-  bad_b = bad[2 * f + 1] != 0;
 #pragma unroll
   for (int k = 0; k < 16; ++k) {
     const int i = t + k * P::T;
     if (i > 0) v[k] = csub(v[k], sh[padded(i - 1)]);
-    if (bad_a) v[k].x = 0.f;
-    if (bad_b) v[k].y = 0.f;
+    size.add(v[k]);
   }
-  __syncthreads();
+  size = row_size<LOGN>(size, part[f], t);
+  const float2 lim = size.limit(nu);
+  const bool mine = !(__uint_as_float(size.ma) <= lim.x && __uint_as_float(size.mb) <= lim.y && size.x.x < kHuge && size.x.y < kHuge);
+  const bool with_large = P::per_block > 1 ? __syncthreads_or(mine) : mine;
+  float2 sum = size.x;
+  if (with_large) {
+    sum = take_large<LOGN>(sh, large + f, part[f], sum, nu, t);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) v[k] = sh[padded(t + k * P::T)];
+  }
+  const int ea = max(__float_as_int(sum.x) >> 23, 1), eb = max(__float_as_int(sum.y) >> 23, 1);
+  if (ea != eb || sum.x == 0.f || sum.y == 0.f) {
+    const float fa = __int_as_float((254 - ea) << 23), fb = __int_as_float((254 - eb) << 23);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) v[k] = make_float2(v[k].x * fa, v[k].y * fb);
+  }
   dft<16, false>(v);
   const float2 w = __ldg(tw + t);
   twiddle<16, false>(v, w);
@@ -254,28 +427,23 @@ __global__ void __launch_bounds__(Plan<LOGN>::threads) k_ramp_filter(const float
   for (int k = 0; k < 16; ++k) v[k] = sh[padded(t + k * P::T)];
   twiddle<16, true>(v, w);
   dft<16, true>(v);
-  const float h0 = 0.25f / (du * du), c = 1.f / (9.8696044f * du * du);
+  if (ea != eb || sum.x == 0.f || sum.y == 0.f) {  // an empty row stays empty
+    const float fa = sum.x == 0.f ? 0.f : __int_as_float(ea << 23), fb = sum.y == 0.f ? 0.f : __int_as_float(eb << 23);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) v[k] = make_float2(v[k].x * fa, v[k].y * fb);
+  }
 #pragma unroll
   for (int row = 0; row < 2; ++row) {
     const int r = r0 + row;
     if (r >= rows) continue;
-    const bool direct = row ? bad_b : bad_a;
 #pragma unroll
     for (int k = 0; k < 16; ++k) {
       const int i = t + k * P::T;
-      if (i >= nu) continue;
-      float o = row ? v[k].y : v[k].x;
-      if (direct) {
-        float acc = 0.f;
-        for (int j = 0; j < nu; ++j) {
-          const int d = i - j;
-          const float h = d == 0 ? h0 : ((d & 1) ? -c / ((float)d * (float)d) : 0.f);
-          acc = fmaf(weighted(__ldg(p + (size_t)r * nu + j), row ? vb : va, j), h, acc);
-        }
-        o = acc * du;
-      }
-      q[(size_t)r * nu + i] = o;
+      if (i < nu) q[(size_t)r * nu + i] = row ? v[k].y : v[k].x;
     }
+    if (with_large)
+      add_large<LOGN>(p + (size_t)r * nu, q + (size_t)r * nu, large[f].pixel[row], large[f].step[row], ramp, nu, du,
+                      row ? vb : va, sod, t);
   }
 }
 
@@ -297,7 +465,7 @@ cudaError_t launch(const float* p, int nu, int nv, int rows, float du, float dv,
   }
   const int pairs = (rows + 1) / 2;
   k_ramp_filter<LOGN><<<(pairs + P::per_block - 1) / P::per_block, P::threads, smem, s>>>(p, nu, nv, rows, du, dv, sod,
-                                                                                          tw, spec, q);
+                                                                                          ramp, tw, spec, q);
   return cudaGetLastError();
 }
 
