@@ -61,13 +61,16 @@ __global__ void k_sg_cols(const float* __restrict__ in, float* __restrict__ out,
   }
 }
 
-// Keys cubic convolution weights for taps at offsets -1, 0, 1, 2 from floor(x).
+// Keys cubic convolution weights for taps at offsets -1, 0, 1, 2 from floor(x); the multiply-adds are written out, so
+// that every place that inlines this gets the same bits.
 __device__ __forceinline__ void keys_weights(float t, float a, float wt[4]) {
   const float d0 = 1.f + t, d1 = t, d2 = 1.f - t, d3 = 2.f - t;
-  wt[0] = ((a * d0 - 5.f * a) * d0 + 8.f * a) * d0 - 4.f * a;
-  wt[1] = ((a + 2.f) * d1 - (a + 3.f)) * d1 * d1 + 1.f;
-  wt[2] = ((a + 2.f) * d2 - (a + 3.f)) * d2 * d2 + 1.f;
-  wt[3] = ((a * d3 - 5.f * a) * d3 + 8.f * a) * d3 - 4.f * a;
+  auto outer = [a](float d) { return fmaf(fmaf(fmaf(a, d, -5.f * a), d, 8.f * a), d, -4.f * a); };
+  auto inner = [a](float d) { return fmaf(fmaf(a + 2.f, d, -(a + 3.f)) * d, d, 1.f); };
+  wt[0] = outer(d0);
+  wt[1] = inner(d1);
+  wt[2] = inner(d2);
+  wt[3] = outer(d3);
 }
 
 // out[o][Y][X] = sum_ty sum_tx wy wx ((1-f) in[a0][y][x] + f in[a1][y][x]),
