@@ -160,10 +160,12 @@ __device__ __forceinline__ void middle(float2* sh, int t, const float2* tw, cons
   __syncthreads();
 }
 
-// W^k = exp(-2 pi i k / N)
-__global__ void k_ramp_twiddles(int n, float2* __restrict__ tw) {
+// W^k = exp(-2 pi i k / N), and the taps h(d) at d mod N, as the direct sum takes them
+__global__ void k_ramp_twiddles(int n, float du, float2* __restrict__ tw, float* __restrict__ taps) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n) return;
+  const int d = min(k, n - k);
+  taps[k] = d == 0 ? 0.25f / (du * du) : ((d & 1) ? -(1.f / (9.8696044f * du * du)) / ((float)d * (float)d) : 0.f);
   float s, c;
   sincospif(2.f * (float)k / (float)n, &s, &c);
   tw[k] = make_float2(c, -s);
@@ -320,28 +322,27 @@ __device__ __noinline__ float2 take_large(float2* sh, Large<LOGN>* large, RowSiz
 }
 
 // Adds what the large pixels and differences of a row (p, at height v) contribute to the outputs that this thread stored
-// in q; gs: G, see ramp_kernel.
+// in q; gs, hs: G(d) and h(d) at d mod N (one load and one multiply-add per tap: an object 50 pixels wide, whose every
+// pixel is a large one, costs as much again as the transform).
 template <int LOGN>
 __device__ __noinline__ void add_large(const float* __restrict__ p, float* __restrict__ q, const uint32_t* pixel,
-                                       const uint32_t* step, const float* __restrict__ gs, int nu, float du, float v,
-                                       float sod, int t) {
+                                       const uint32_t* step, const float* __restrict__ gs,
+                                       const float* __restrict__ hs, int nu, float du, float v, float sod, int t) {
   using P = Plan<LOGN>;
   uint32_t any = 0u;
   for (int k = 0; k < Large<LOGN>::words; ++k) any |= pixel[k] | step[k];
   if (!any) return;
-  const float h0 = 0.25f / (du * du), c = 1.f / (9.8696044f * du * du);
   float acc[16] = {};
-  for (int b = 0; b < Large<LOGN>::words; ++b) {
-    for (uint32_t m = pixel[b]; m; m &= m - 1) {
+  bool nan = false;  // then so is every output
+  for (int b = 0; b < Large<LOGN>::words && !nan; ++b) {
+    for (uint32_t m = pixel[b]; m && !nan; m &= m - 1) {
       const int j = 32 * b + __ffs(m) - 1;
       const float x = weighted(__ldg(p + j), v, j, nu, du, sod);
 #pragma unroll
-      for (int k = 0; k < 16; ++k) {
-        const int d = t + k * P::T - j;
-        acc[k] = fmaf(x, d == 0 ? h0 : ((d & 1) ? -c / ((float)d * (float)d) : 0.f), acc[k]);
-      }
+      for (int k = 0; k < 16; ++k) acc[k] = fmaf(x, __ldg(hs + ((t + k * P::T - j) & (P::N - 1))), acc[k]);
+      nan = x != x;
     }
-    for (uint32_t m = step[b]; m; m &= m - 1) {
+    for (uint32_t m = nan ? 0u : step[b]; m; m &= m - 1) {
       const int j = 32 * b + __ffs(m) - 1;
       auto at = [&](int i) -> float {  // the row without its large pixels
         return i < 0 || i >= nu || ((pixel[i >> 5] >> (i & 31)) & 1u) ? 0.f : weighted(__ldg(p + i), v, i, nu, du, sod);
@@ -358,7 +359,7 @@ __device__ __noinline__ void add_large(const float* __restrict__ p, float* __res
   }
 }
 
-// Filters rows 2 b and 2 b + 1 (b the transform's number); ramp, tw, g: see launch.
+// Filters rows 2 b and 2 b + 1 (b the transform's number); ramp: G, then tw, the spectrum g and the taps.
 template <int LOGN>
 __global__ void __launch_bounds__(Plan<LOGN>::threads) k_ramp_filter(const float* __restrict__ p, int nu, int nv,
                                                                      int rows, float du, float dv, float sod,
@@ -442,8 +443,8 @@ __global__ void __launch_bounds__(Plan<LOGN>::threads) k_ramp_filter(const float
       if (i < nu) q[(size_t)r * nu + i] = row ? v[k].y : v[k].x;
     }
     if (with_large)
-      add_large<LOGN>(p + (size_t)r * nu, q + (size_t)r * nu, large[f].pixel[row], large[f].step[row], ramp, nu, du,
-                      row ? vb : va, sod, t);
+      add_large<LOGN>(p + (size_t)r * nu, q + (size_t)r * nu, large[f].pixel[row], large[f].step[row], ramp,
+                      ramp + 5 * P::N, nu, du, row ? vb : va, sod, t);
   }
 }
 
@@ -460,7 +461,7 @@ cudaError_t launch(const float* p, int nu, int nv, int rows, float du, float dv,
   }
   float2 *tw = reinterpret_cast<float2*>(ramp + P::N), *spec = tw + P::N;
   if (tables) {
-    k_ramp_twiddles<<<(P::N + 255) / 256, 256, 0, s>>>(P::N, tw);
+    k_ramp_twiddles<<<(P::N + 255) / 256, 256, 0, s>>>(P::N, du, tw, ramp + 5 * P::N);
     k_ramp_spectrum<LOGN><<<1, P::threads, smem, s>>>(ramp, du / (float)P::N, tw, spec);
   }
   const int pairs = (rows + 1) / 2;

@@ -1322,7 +1322,7 @@ int mc_fdk(mc_ctx* ctx, const float* p, int n_proj, const float* angles, int NU,
   const size_t img = (size_t)NU * NV;
   const size_t room = std::max(kFdkChunk / 4, (size_t)nx * ny * nz);
   const int chunk = (int)std::max<size_t>(1, std::min<size_t>((size_t)n_proj, room / img));
-  const size_t table = cs.size() + 4 * (size_t)points;
+  const size_t table = cs.size() + 5 * (size_t)points;
   CK(ensure(ctx->d_fdk, ctx->fdk_cap, table + chunk * img), "fdk allocation");
   float* d_cs = ctx->d_fdk;
   cudaError_t e = cudaMemcpyAsync(d_cs, cs.data(), cs.size() * 4, cudaMemcpyHostToDevice, s);

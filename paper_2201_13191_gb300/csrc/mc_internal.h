@@ -238,7 +238,7 @@ int wgrad_splits(int n, int h, int w, int cin, int cout);
 cudaError_t recon_log_norm(const float* I, const float* I0, size_t img, size_t n, float* a, cudaStream_t s);
 // Ramp filter by transforms (k_ramp.cu): ramp_points: transform length for rows of nu values (0: rows longer than
 // 4096, filtered by direct sums); ramp_kernel: the summed kernel (host, ramp_points values); ramp: device, the summed
-// kernel followed by 4 ramp_points floats, the tables, which are made when `tables` is set.
+// kernel followed by 5 ramp_points floats, the tables, which are made when `tables` is set.
 int ramp_points(int nu);
 void ramp_kernel(int nu, float du, float* g);
 cudaError_t ramp_filter(const float* p, int nu, int nv, int rows, float du, float dv, float sod, float* ramp, float* q,
