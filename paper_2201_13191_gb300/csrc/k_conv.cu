@@ -344,9 +344,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv3x3_fwd(const __grid_consta
 // separate MMAs of NT columns (the 15 layers of one step: 1030 -> 690 us), and neither
 // operand passes through registers.  In the image's first and last row the MMA
 // leaves out the columns of the dy that falls outside, so that a value that is
-// not finite meets the same products as in the sum above; only where the width is
-// no multiple of 16 can one in the last column reach its dx = -1 tap too (and
-// in 8-wide tiles one in the first or last row its third dy).
+// not finite meets the same products as in the sum above.  Where the width is no
+// multiple of 16 such a value also meets the zeros beside the image (in the last
+// column's dx = -1; in 8-wide tiles in the first or last row's third dy): there
+// the accumulators that are not finite are summed again from global memory.
 //
 // CTA (cin chunk, cout tile, split): the split's tiles, a run of neighbours (its
 // partial sums then grow, and round, like those of a run of pixels), go through a
@@ -378,11 +379,35 @@ struct WgPlan {
 
 struct WgArgs {
   float* dw;
-  int n, h, w, cin, tx, ty, tiles_x, tiles_y;  // tx x ty: the tile
+  const __nv_bfloat16 *x, *dy;
+  int n, h, w, cin, cout, tx, ty, tiles_x, tiles_y;  // tx x ty: the tile
   int* err;
 };
 
-template <int CC, int NT>
+// dW[co][tap_y, tap_x][c] over `count` tiles from `first` on, the products inside the image only.
+__device__ __noinline__ float wgrad_direct(WgArgs p, long long first, int count, int c, int co, int tap_y, int tap_x) {
+  const int per_img = p.tiles_x * p.tiles_y;
+  float sum = 0.f;
+  for (long long t = first; t < first + count; ++t) {
+    const long long img = t / per_img;
+    const int r = (int)(t - img * per_img), y0 = (r / p.tiles_x) * p.ty, x0 = (r % p.tiles_x) * p.tx;
+    for (int y = y0; y < min(y0 + p.ty, p.h); ++y) {
+      const int gy = y - (tap_y - 1);
+      if (gy < 0 || gy >= p.h) continue;
+      const __nv_bfloat16* row_x = p.x + (img * p.h + y) * p.w * p.cin + c;
+      const __nv_bfloat16* row_g = p.dy + (img * p.h + gy) * p.w * p.cout + co;
+      for (int x = x0; x < min(x0 + p.tx, p.w); ++x) {
+        const int px = x + tap_x - 1;
+        if (px >= 0 && px < p.w)
+          sum = fmaf(__bfloat162float(row_x[(long long)px * p.cin]), __bfloat162float(row_g[(long long)x * p.cout]), sum);
+      }
+    }
+  }
+  return sum;
+}
+
+// RAGGED: the width is no multiple of 16 (a variant of its own: the sums from global memory double the registers).
+template <int CC, int NT, bool RAGGED>
 __global__ void __launch_bounds__(kThreads) k_conv3x3_wgrad(const __grid_constant__ CUtensorMap xmap,
                                                             const __grid_constant__ CUtensorMap ymap, const WgArgs p) {
   using P = WgPlan<CC, NT>;
@@ -482,18 +507,52 @@ __global__ void __launch_bounds__(kThreads) k_conv3x3_wgrad(const __grid_constan
   if (ok && count > 0) {
     // accumulator row = block of CC channels (dx) x channel
     const int m = warp * 32 + lane, c = m % CC, blk = m / CC;
+    auto tap = [&](int a) { return 3 * (2 - a % 3) + blk + 2 * (a / 3); };  // of accumulator a, where blk + 2 (a / 3) < 3
+    bool again = false;
+    if constexpr (RAGGED) {
+      // a pass of its own: with the test inside the loop of the adds the 64 x 64 form takes 44 us instead of 39 (mean of the 208^2 layers)
+      constexpr int step = NT >= 32 ? 32 : 8;
 #pragma unroll 1
-    for (int a = 0; a < 3 * P::groups; ++a) {
-      const int dy = 2 - a % 3, dx = blk + 2 * (a / 3);
-      const bool use = dx < 3;
-      float* dst = p.dw + (size_t)n0 * 9 * p.cin + (size_t)(3 * dy + dx) * p.cin + c0 + c;
-#pragma unroll 1
-      for (int j0 = 0; j0 < NT; j0 += 8) {
-        float v[8];
-        tc::tmem_ld8(lane_base + (uint32_t)(a * NT + j0), v);
-        if (use)
+      for (int j0 = 0; j0 < P::cols; j0 += step) {
+        float v[step], z = 0.f;  // z: no number if one of v is not finite
+        if constexpr (step == 32) tc::tmem_ld32(lane_base + (uint32_t)j0, v);
+        else tc::tmem_ld8(lane_base + (uint32_t)j0, v);
 #pragma unroll
-          for (int j = 0; j < 8; ++j) atomicAdd(dst + (size_t)(j0 + j) * 9 * p.cin, v[j]);
+        for (int j = 0; j < step; j += 4) z += fmaf(v[j], 0.f, v[j + 1] * 0.f) + fmaf(v[j + 2], 0.f, v[j + 3] * 0.f);
+        again |= blk + 2 * (j0 / (3 * NT)) < 3 && z != 0.f;
+      }
+      again = __any_sync(0xFFFFFFFFu, again);
+    }
+    if (RAGGED && again) {
+#pragma unroll 1
+      for (int j = 0; j < P::cols; j += 8) {
+        float v[8];
+        __syncwarp();
+        tc::tmem_ld8(lane_base + (uint32_t)j, v);
+        const int a = j / NT, n = n0 + j % NT;
+        if (blk + 2 * (a / 3) >= 3) continue;
+#pragma unroll 1
+        for (int i = 0; i < 8; ++i) {
+          float o = v[0];
+#pragma unroll
+          for (int q = 1; q < 8; ++q) o = q == i ? v[q] : o;
+          if (!(fabsf(o) < INFINITY)) o = wgrad_direct(p, first, count, c0 + c, n + i, tap(a) / 3, tap(a) % 3);
+          atomicAdd(p.dw + ((size_t)(n + i) * 9 + tap(a)) * p.cin + c0 + c, o);
+        }
+      }
+    } else {
+#pragma unroll 1
+      for (int a = 0; a < 3 * P::groups; ++a) {
+        const bool use = blk + 2 * (a / 3) < 3;
+        float* dst = p.dw + (size_t)n0 * 9 * p.cin + (size_t)tap(a) * p.cin + c0 + c;
+#pragma unroll 1
+        for (int j0 = 0; j0 < NT; j0 += 8) {
+          float v[8];
+          tc::tmem_ld8(lane_base + (uint32_t)(a * NT + j0), v);
+          if (use)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) atomicAdd(dst + (size_t)(j0 + j) * 9 * p.cin, v[j]);
+        }
       }
     }
   }
@@ -699,17 +758,21 @@ cudaError_t launch_wgrad_n(const WgradParams& p, int splits, cudaStream_t s) {
   if (!nhwc_map(enc, &xmap, p.x, p.n, p.h, p.w, p.cin, CC, a.tx + 2, a.ty) ||
       !nhwc_map(enc, &ymap, p.dy, p.n, p.h, p.w, p.cout, NT, a.tx, a.ty + 2))
     return cudaErrorInvalidValue;
-  cudaError_t e = cudaFuncSetAttribute(k_conv3x3_wgrad<CC, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, P::smem);
+  auto* k = p.w % 16 ? k_conv3x3_wgrad<CC, NT, true> : k_conv3x3_wgrad<CC, NT, false>;
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, P::smem);
   if (e != cudaSuccess) return e;
   a.dw = p.dw;
+  a.x = p.x;
+  a.dy = p.dy;
   a.n = p.n;
   a.h = p.h;
   a.w = p.w;
   a.cin = p.cin;
+  a.cout = p.cout;
   a.tiles_x = (p.w + a.tx - 1) / a.tx;
   a.tiles_y = (p.h + a.ty - 1) / a.ty;
   a.err = p.err;
-  k_conv3x3_wgrad<CC, NT><<<dim3(p.cin / CC, p.cout / NT, splits), kThreads, P::smem, s>>>(xmap, ymap, a);
+  k<<<dim3(p.cin / CC, p.cout / NT, splits), kThreads, P::smem, s>>>(xmap, ymap, a);
   return cudaGetLastError();
 }
 
