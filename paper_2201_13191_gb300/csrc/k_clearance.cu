@@ -135,12 +135,6 @@ __global__ void __launch_bounds__(1024) k_palette(const uint32_t* __restrict__ s
     }
 }
 
-// What makes two voxels the same: the palette index, or the voxel word.
-template <int LAYOUT>
-__device__ __forceinline__ uint32_t entry(const uint32_t* __restrict__ vox, size_t i) {
-  return __ldg(vox + (LAYOUT == VOX_HOP2 ? 2 * i : i));
-}
-
 // Palette indices, or voxel words beside an empty word, over the padded grid (border voxels repeat the nearest edge
 // voxel).
 template <int LAYOUT>
@@ -161,15 +155,17 @@ __global__ void __launch_bounds__(256) k_pack_clearance(const uint8_t* __restric
   }
 }
 
-// Level 1: cell (x, y, z) is uniform; cells past the last voxel compare the
+// Level 1 over the padded grid, from the volume's own arrays, so that a volume is looked over before any words are made
+// for it: cell (x, y, z) is uniform; cells past the last voxel compare the
 // voxels there are, bits past the row are set.  Counts the mixed cells.  A warp
 // walks kZRun planes of one row word: a plane's 2 x 2 patch is reduced to its
 // value (or "mixed") once and serves the cells below and above it, with the
-// x + 1 neighbours from a shuffle: 2 loads per voxel.
+// x + 1 neighbours from a shuffle: 2 voxels read per voxel.
 constexpr int kZRun = 8;
-template <int LAYOUT>
-__global__ void __launch_bounds__(256) k_cells(const uint32_t* __restrict__ vox, int px, int py, int pz, int wpr,
-                                               uint32_t* __restrict__ bits, unsigned long long* mixed) {
+__global__ void __launch_bounds__(256) k_cells(const uint8_t* __restrict__ mat, const uint16_t* __restrict__ rho, int nx,
+                                               int ny, int nz, int wpr, uint32_t* __restrict__ bits,
+                                               unsigned long long* mixed) {
+  const int px = nx + 2, py = ny + 2, pz = nz + 2;
   const uint32_t runs = (uint32_t)((pz + kZRun - 1) / kZRun);
   const uint32_t work = (uint32_t)wpr * (uint32_t)py * runs;
   const int lane = threadIdx.x & 31;
@@ -177,15 +173,18 @@ __global__ void __launch_bounds__(256) k_cells(const uint32_t* __restrict__ vox,
   for (uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < work; i += (gridDim.x * blockDim.x) >> 5) {
     const uint32_t t = i / (uint32_t)wpr, wi = i - t * (uint32_t)wpr;
     const int y = (int)(t % (uint32_t)py), z0 = (int)(t / (uint32_t)py) * kZRun, z1 = min(z0 + kZRun, pz);
-    const int x = (int)wi * 32 + lane, xc = min(x, px - 1), xe = min(x + 1, px - 1), y1 = min(y + 1, py - 1);
-    constexpr uint32_t kMixed = 0xFFFFFFFFu;  // no palette index, no voxel word
+    // border voxels repeat the nearest edge voxel
+    const int x = (int)wi * 32 + lane, xc = min(max(x - 1, 0), nx - 1), xe = min(x, nx - 1);
+    const int y0 = min(max(y - 1, 0), ny - 1), y1 = min(y, ny - 1);
+    constexpr uint32_t kMixed = 0xFFFFFFFFu;  // no voxel's key
+    auto key = [&](size_t at) { return voxel_key(__ldg(mat + at), __ldg(rho + at)); };
     auto patch = [&](int z) -> uint32_t {
-      const size_t r0 = ((size_t)z * py + y) * px, r1 = ((size_t)z * py + y1) * px;
-      const uint32_t a = entry<LAYOUT>(vox, r0 + xc), b = entry<LAYOUT>(vox, r1 + xc);
+      const size_t zs = (size_t)min(max(z - 1, 0), nz - 1) * ny, r0 = (zs + y0) * nx, r1 = (zs + y1) * nx;
+      const uint32_t a = key(r0 + xc), b = key(r1 + xc);
       uint32_t an = __shfl_down_sync(0xffffffffu, a, 1), bn = __shfl_down_sync(0xffffffffu, b, 1);
       if (lane == 31) {
-        an = entry<LAYOUT>(vox, r0 + xe);
-        bn = entry<LAYOUT>(vox, r1 + xe);
+        an = key(r0 + xe);
+        bn = key(r1 + xe);
       }
       return a == b && a == an && a == bn ? a : kMixed;
     };
@@ -335,6 +334,9 @@ cudaError_t read_scan(void* scratch, VolumeScan* out, cudaStream_t s) {
 }  // namespace
 
 size_t scan_scratch_bytes() { return kScanBytes + kKeys / 8 + kKeys; }
+size_t cells_scratch_bytes(int nx, int ny, int nz) {
+  return scan_scratch_bytes() + level_words(nx + 2, ny + 2, nz + 2) * 4;
+}
 size_t clearance_scratch_bytes(int nx, int ny, int nz) {
   return scan_scratch_bytes() + (size_t)kLevels * level_words(nx + 2, ny + 2, nz + 2) * 4;
 }
@@ -356,35 +358,30 @@ cudaError_t scan_volume(const uint8_t* mat, const uint16_t* rho, int nx, int ny,
   return e == cudaSuccess ? read_scan(scratch, out, s) : e;
 }
 
-cudaError_t pack_clearance(const uint8_t* mat, const uint16_t* rho, int nx, int ny, int nz, int layout, void* scratch,
-                           uint32_t* vox, double* mixed, cudaStream_t s) {
-  VolumeView v;
-  padded_dims(nx, ny, nz, layout, &v);
-  const int wpr = (v.px + 31) / 32;
+cudaError_t mixed_cells(const uint8_t* mat, const uint16_t* rho, int nx, int ny, int nz, void* scratch, double* share,
+                        cudaStream_t s) {
+  const int wpr = (nx + 2 + 31) / 32;
   auto* scan = static_cast<VolumeScan*>(scratch);
   cudaError_t e = cudaMemsetAsync(&scan->mixed, 0, sizeof(scan->mixed), s);
   if (e != cudaSuccess) return e;
-  const int g = grid_of((size_t)v.words), gc = grid_of(level_words(v.px, v.py, (v.pz + kZRun - 1) / kZRun) * 32);
-  if (layout == VOX_HOP2) {
-    k_pack_clearance<VOX_HOP2><<<g, 256, 0, s>>>(mat, rho, v, scratch_map(scratch), vox);
-    k_cells<VOX_HOP2><<<gc, 256, 0, s>>>(vox, v.px, v.py, v.pz, wpr, scratch_levels(scratch), &scan->mixed);
-  } else {
-    k_pack_clearance<VOX_HOP><<<g, 256, 0, s>>>(mat, rho, v, scratch_map(scratch), vox);
-    k_cells<VOX_HOP><<<gc, 256, 0, s>>>(vox, v.px, v.py, v.pz, wpr, scratch_levels(scratch), &scan->mixed);
-  }
+  k_cells<<<grid_of(level_words(nx + 2, ny + 2, (nz + 2 + kZRun - 1) / kZRun) * 32), 256, 0, s>>>(
+      mat, rho, nx, ny, nz, wpr, scratch_levels(scratch), &scan->mixed);
   e = cudaGetLastError();
   VolumeScan h = {};
   if (e == cudaSuccess) e = read_scan(scratch, &h, s);
-  *mixed = (double)h.mixed / (double)v.words;
+  *share = (double)h.mixed / ((double)(nx + 2) * (ny + 2) * (nz + 2));
   return e;
 }
 
-cudaError_t build_clearance(int nx, int ny, int nz, int layout, void* scratch, uint32_t* vox, cudaStream_t s) {
+cudaError_t build_clearance(const uint8_t* mat, const uint16_t* rho, int nx, int ny, int nz, int layout, void* scratch,
+                            uint32_t* vox, cudaStream_t s) {
   VolumeView v;
   padded_dims(nx, ny, nz, layout, &v);
   uint32_t* bits = scratch_levels(scratch);
   const size_t lw = level_words(v.px, v.py, v.pz);
-  const int wpr = (v.px + 31) / 32;
+  const int wpr = (v.px + 31) / 32, gp = grid_of((size_t)v.words);
+  if (layout == VOX_HOP2) k_pack_clearance<VOX_HOP2><<<gp, 256, 0, s>>>(mat, rho, v, scratch_map(scratch), vox);
+  else k_pack_clearance<VOX_HOP><<<gp, 256, 0, s>>>(mat, rho, v, scratch_map(scratch), vox);
   for (int l = 0; l + 1 < kLevels; ++l)
     k_level<<<grid_of(lw), 256, 0, s>>>(bits + l * lw, (2 << l) - 1, v.py, v.pz, wpr, bits + (l + 1) * lw);
   const size_t blocks = (lw + 32 * kCodeWarps - 1) / (32 * kCodeWarps);

@@ -52,12 +52,12 @@ struct mc_ctx {
   float mesh_half[3] = {0.f, 0.f, 0.f};  // half extents of a box about the origin holding every vertex
   // volume
   bool have_volume = false;
-  uint32_t* d_vox = nullptr;
-  uint32_t* d_hop = nullptr;        // words with clearance (the other layouts: d_vox)
+  uint32_t* d_vox = nullptr;        // packed voxel words (material | FP16 density)
+  uint32_t* d_hop = nullptr;        // words with clearance, while a march uses them
   size_t hop_cap = 0;
   uint32_t* d_pal = nullptr;        // palette of a volume with clearance [kMaxPalette]
   unsigned char* d_prep = nullptr;  // scratch of the volume load
-  size_t pal_cap = 0, prep_cap = 0;  // packed voxel words (material | FP16 density)
+  size_t pal_cap = 0, prep_cap = 0;
   size_t vox_cap = 0;
   int layout = VOX_LIN, layout_p = VOX_LIN;  // of the transport and of the primary
   int nx = 0, ny = 0, nz = 0;
@@ -147,6 +147,18 @@ cudaError_t ensure(T*& p, size_t& cap, size_t n) {
   cudaError_t e = cudaMalloc((void**)&p, n * sizeof(T));
   if (e == cudaSuccess) cap = n;
   return e;
+}
+
+// Gives back what a context keeps between calls and a volume load, which replaces the volume, can do without.
+void drop_kept(mc_ctx* c) {
+  cudaFree(c->d_hop);
+  cudaFree(c->d_prep);
+  cudaFree(c->d_vox);
+  cudaFree(c->d_fdk);
+  c->d_hop = c->d_vox = nullptr;
+  c->d_prep = nullptr;
+  c->d_fdk = nullptr;
+  c->hop_cap = c->prep_cap = c->vox_cap = c->fdk_cap = 0;
 }
 
 // Whether `bytes` from p on lie in one allocation on this device (else, or where it cannot be told: false).
@@ -895,11 +907,15 @@ int mc_load_volume(mc_ctx* ctx, const uint8_t* mat, const uint16_t* rho_fp16, in
   };
   if (!is_device_ptr || ((uintptr_t)rho_fp16 & 1) || !within_allocation(ctx->device, mat, n) ||
       !within_allocation(ctx->device, rho_fp16, n * 2)) {
-    e = cudaMallocAsync((void**)&st_mat, n, s);
-    if (e == cudaSuccess) e = cudaMallocAsync((void**)&st_rho, n * 2, s);
-    if (e != cudaSuccess) {
+    for (bool again = false;; again = true) {
+      e = cudaMallocAsync((void**)&st_mat, n, s);
+      if (e == cudaSuccess) e = cudaMallocAsync((void**)&st_rho, n * 2, s);
+      if (e == cudaSuccess) break;
       release();
-      return cuda_fail(ctx, e, "volume staging allocation");
+      st_mat = nullptr;
+      if (again) return cuda_fail(ctx, e, "volume staging allocation");
+      (void)cudaGetLastError();
+      drop_kept(ctx);
     }
     const cudaMemcpyKind kind = is_device_ptr ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     e = cudaMemcpyAsync(st_mat, mat, n, kind, s);
@@ -913,7 +929,10 @@ int mc_load_volume(mc_ctx* ctx, const uint8_t* mat, const uint16_t* rho_fp16, in
   }
   // one pass: validity (host arrays were checked above), material changes, distinct (material, density) pairs
   VolumeScan scan = {};
-  e = ensure(ctx->d_prep, ctx->prep_cap, scan_scratch_bytes());
+  bool room = ctx->opt.voxel_layout != 2 &&
+              ensure(ctx->d_prep, ctx->prep_cap, cells_scratch_bytes(nx, ny, nz)) == cudaSuccess;
+  (void)cudaGetLastError();
+  if (!room) e = ensure(ctx->d_prep, ctx->prep_cap, scan_scratch_bytes());
   if (e == cudaSuccess) e = ensure(ctx->d_pal, ctx->pal_cap, (size_t)kMaxPalette);
   if (e == cudaSuccess) e = scan_volume(mat, rho_fp16, nx, ny, nz, ctx->n_mat, ctx->d_prep, ctx->d_pal, &scan, s);
   if (e != cudaSuccess || scan.bad) {
@@ -930,39 +949,51 @@ int mc_load_volume(mc_ctx* ctx, const uint8_t* mat, const uint16_t* rho_fp16, in
   const size_t plain_bytes = packed_words(nx, ny, nz, VOX_LIN) * 4;
   int layout = ctx->opt.voxel_layout == 2 ? VOX_BRICK : VOX_LIN;
   int layout_p = -1;
-  if (e == cudaSuccess && layout != VOX_BRICK) {
+  if (e == cudaSuccess && room) {
     const int hop = scan.pairs <= (uint32_t)kMaxPalette ? VOX_HOP : VOX_HOP2;
-    const size_t words = packed_words(nx, ny, nz, hop), need = clearance_scratch_bytes(nx, ny, nz);
-    // without room for the larger words or the scratch the volume is packed plainly
-    bool room = words <= ctx->hop_cap || ensure(ctx->d_hop, ctx->hop_cap, words) == cudaSuccess;
-    if (room && need > ctx->prep_cap) {
-      unsigned char* larger = nullptr;
-      room = cudaMalloc((void**)&larger, need) == cudaSuccess;
-      if (room) {
-        // the scan's results stay
-        e = cudaMemcpyAsync(larger, ctx->d_prep, scan_scratch_bytes(), cudaMemcpyDeviceToDevice, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        cudaFree(ctx->d_prep);
-        ctx->d_prep = larger;
-        ctx->prep_cap = need;
+    const MixedLimits lim = mixed_limits(plain_bytes, (size_t)l2);
+    double mixed = 1.0;
+    e = mixed_cells(mat, rho_fp16, nx, ny, nz, ctx->d_prep, &mixed, s);
+    // without room for the larger words or their scratch the volume is packed plainly
+    if (e == cudaSuccess && mixed <= lim.primary) {
+      room = ensure(ctx->d_hop, ctx->hop_cap, packed_words(nx, ny, nz, hop)) == cudaSuccess;
+      const size_t need = clearance_scratch_bytes(nx, ny, nz), have = cells_scratch_bytes(nx, ny, nz);
+      if (room && need > ctx->prep_cap) {
+        unsigned char* larger = nullptr;
+        room = cudaMalloc((void**)&larger, need) == cudaSuccess;
+        if (room) {
+          // what the scan and the cells left stays
+          e = cudaMemcpyAsync(larger, ctx->d_prep, have, cudaMemcpyDeviceToDevice, s);
+          if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+          cudaFree(ctx->d_prep);
+          ctx->d_prep = larger;
+          ctx->prep_cap = need;
+        }
       }
-    }
-    if (!room) (void)cudaGetLastError();
-    if (room && e == cudaSuccess) {
-      double mixed = 1.0;
-      e = pack_clearance(mat, rho_fp16, nx, ny, nz, hop, ctx->d_prep, ctx->d_hop, &mixed, s);
-      const MixedLimits lim = mixed_limits(plain_bytes, (size_t)l2);
-      if (e == cudaSuccess && mixed <= lim.primary) {
+      if (!room) (void)cudaGetLastError();
+      if (room && e == cudaSuccess) {
         layout_p = hop;
         if (mixed <= lim.transport) layout = hop;
-        e = build_clearance(nx, ny, nz, hop, ctx->d_prep, ctx->d_hop, s);
+        e = build_clearance(mat, rho_fp16, nx, ny, nz, hop, ctx->d_prep, ctx->d_hop, s);
       }
     }
+  }
+  if (layout_p < 0 && ctx->d_hop) {
+    cudaFree(ctx->d_hop);
+    ctx->d_hop = nullptr;
+    ctx->hop_cap = 0;
   }
   if (e == cudaSuccess && !is_hop(layout)) {
     if (ctx->opt.voxel_layout == 0 && (double)plain_bytes > 0.75 * (double)l2) layout = VOX_BRICK;
     const size_t words = packed_words(nx, ny, nz, layout);
     e = ensure(ctx->d_vox, ctx->vox_cap, words);
+    if (e == cudaErrorMemoryAllocation) {
+      // the plain words come first
+      (void)cudaGetLastError();
+      drop_kept(ctx);
+      layout_p = -1;
+      e = ensure(ctx->d_vox, ctx->vox_cap, words);
+    }
     if (e == cudaSuccess) e = pack_volume(mat, rho_fp16, nx, ny, nz, layout, ctx->d_vox, words, s);
   }
   release();

@@ -193,13 +193,16 @@ constexpr int kMaxPalette = 256;
 size_t scan_scratch_bytes();
 cudaError_t scan_volume(const uint8_t* mat, const uint16_t* rho, int nx, int ny, int nz, int n_mat, void* scratch,
                         uint32_t* pal, VolumeScan* out, cudaStream_t s);
-// Volumes with clearance (layout VOX_HOP from a scan that found at most kMaxPalette pairs, or VOX_HOP2), scratch of
-// clearance_scratch_bytes: pack_clearance packs the voxels into vox and measures the share of 2x2x2 voxel cells that
-// are mixed (synchronises s); build_clearance adds the octant codes.
+// Volumes with clearance (layout VOX_HOP from a scan that found at most kMaxPalette pairs, or VOX_HOP2), after the scan,
+// in the same scratch: mixed_cells (cells_scratch_bytes of it) measures the share of 2x2x2 voxel cells that are mixed
+// and leaves a bit per cell there (synchronises s); build_clearance (clearance_scratch_bytes) packs the voxels into vox
+// with their octant codes.
+size_t cells_scratch_bytes(int nx, int ny, int nz);
 size_t clearance_scratch_bytes(int nx, int ny, int nz);
-cudaError_t pack_clearance(const uint8_t* mat, const uint16_t* rho, int nx, int ny, int nz, int layout, void* scratch,
-                           uint32_t* vox, double* mixed, cudaStream_t s);
-cudaError_t build_clearance(int nx, int ny, int nz, int layout, void* scratch, uint32_t* vox, cudaStream_t s);
+cudaError_t mixed_cells(const uint8_t* mat, const uint16_t* rho, int nx, int ny, int nz, void* scratch, double* share,
+                        cudaStream_t s);
+cudaError_t build_clearance(const uint8_t* mat, const uint16_t* rho, int nx, int ny, int nz, int layout, void* scratch,
+                            uint32_t* vox, cudaStream_t s);
 // Padded dimensions, brick counts and word count of a packed volume.
 void padded_dims(int nx, int ny, int nz, int layout, VolumeView* v);
 
