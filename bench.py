@@ -45,7 +45,7 @@ def parse():
     p.add_argument("--photons", type=float, default=None, help="override photons per step")
     p.add_argument("--cpu-seconds", type=float, default=12.0, help="oracle sample budget")
     p.add_argument("--no-cpu-baseline", action="store_true")
-    p.add_argument("--voxel-layout", type=int, default=0, help="0 default, 1 linear, 2 4^3 bricks")
+    p.add_argument("--voxel-layout", type=int, default=0, help="0 default (by the volume), 1 x fastest, 2 4^3 bricks")
     p.add_argument("--workload", default=WORKLOAD, help="ell256 (default) or ell512 (batched angles)")
     p.add_argument("--angles", type=int, default=1, help="projection angles per step (one launch)")
     p.add_argument("--per-angle", action="store_true", help="one mc_project call per angle instead of one batch")

@@ -83,9 +83,10 @@ typedef struct mc_options {
   float cubic_a;         /* Keys cubic parameter of the spatial up-sampling, default -0.5 (Sec. II-C.3) */
   int denoise_mode;      /* 0 = Savitzky-Golay, 1 = learned denoiser (mc_denoise_*), 2 = none */
   int voxel_layout;      /* device volume layout: 1 = x fastest, 2 = 4x4x4 Morton bricks, 0 = default:
-                            x fastest while the packed volume fits in 3/4 of L2, bricks beyond.  With 0 and 1 a
-                            volume with large uniform parts is stored x fastest with the uniform cube ahead of
-                            each voxel, which a march takes in one step; the images and counters are the same */
+                            a volume with large uniform parts is stored x fastest with the uniform cube ahead of
+                            each voxel, which a march takes in one step; others x fastest while the packed volume
+                            fits in 3/4 of L2, bricks beyond.  The primary image and the counters are the same in
+                            every layout, the scatter agrees to the FP32 rounding of the rays' optical depths */
   int use_graph;         /* 1: mc_project replays one captured CUDA graph while its launch shape is unchanged */
   int nee_mode;          /* point-detector scoring (Sec. II-C.1): 0 = the sampled scatter type's pdf (the
                             paper's, default); 1 = expected value over the interaction type: every

@@ -929,7 +929,7 @@ int mc_load_volume(mc_ctx* ctx, const uint8_t* mat, const uint16_t* rho_fp16, in
   }
   // one pass: validity (host arrays were checked above), material changes, distinct (material, density) pairs
   VolumeScan scan = {};
-  bool room = ctx->opt.voxel_layout != 2 &&
+  bool room = ctx->opt.voxel_layout == 0 &&
               ensure(ctx->d_prep, ctx->prep_cap, cells_scratch_bytes(nx, ny, nz)) == cudaSuccess;
   (void)cudaGetLastError();
   if (!room) e = ensure(ctx->d_prep, ctx->prep_cap, scan_scratch_bytes());
@@ -940,7 +940,7 @@ int mc_load_volume(mc_ctx* ctx, const uint8_t* mat, const uint16_t* rho_fp16, in
     if (e != cudaSuccess) return cuda_fail(ctx, e, "volume validation");
     return fail(ctx, MC_ERR_INVALID_ARG, "volume holds an unknown material id or an invalid density");
   }
-  // Layout.  Default: words with clearance (x fastest) where few of the volume's cells are mixed, so that a march takes
+  // Layout.  As asked for, or by default: words with clearance (x fastest) where few of the volume's cells are mixed, so that a march takes
   // many midpoints from one word.  Otherwise x fastest while the packed volume fits in 3/4 of L2 (measured faster
   // there), 4^3 bricks once it streams from HBM (every ray direction then reuses its sectors).  The primary gains from
   // clearance up to a larger share of mixed cells than the transport, so a volume may be packed both ways.
