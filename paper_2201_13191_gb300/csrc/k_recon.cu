@@ -120,7 +120,9 @@ __device__ __forceinline__ float div_by(float a, float b, float r) {
 // taps lie close together on the panel whatever the angle (a row of 32 in x
 // spreads over up to 130 panel pixels).  256^3 x 360 projections of 1024^2: 15.3
 // -> 9.3 ms with these tiles, the divisions by a stored reciprocal and ZB = 8.
-template <int ZB>
+// WIDE: projections of 2^31 pixels or more, or more than 2^22 rows, where a
+// pixel's number needs 64 bits and its floor the conversion.
+template <int ZB, bool WIDE>
 __global__ void __launch_bounds__(256) k_fdk_backproject(const float* __restrict__ q, const float* __restrict__ cb,
                                                          const float* __restrict__ sb, int n_proj, int nu, int nv,
                                                          float du_iso, float dv_iso, float inv_du, float inv_dv,
@@ -147,6 +149,14 @@ __global__ void __launch_bounds__(256) k_fdk_backproject(const float* __restrict
     acc[j] = first || iz0 + j >= nz ? 0.f : vol[((size_t)(iz0 + j) * ny + iy) * nx + ix];
   }
   const size_t img = (size_t)nu * nv;
+  // row v0 of q from column u0 on, v0 the floor fw of fv (a round-down add's sum where not WIDE)
+  auto floor_of = [&](float f) { return WIDE ? floorf(f) : __fadd_rd(f, kFloor); };
+  auto fraction = [&](float f, float fl) { return WIDE ? f - fl : f - (fl - kFloor); };
+  auto whole = [&](float fl) { return WIDE ? (int)fl : __float_as_int(fl) - 0x4B400000; };
+  auto row = [&](float fw, int u0) -> const float* {
+    if constexpr (WIDE) return q + ((size_t)whole(fw) * nu + u0);
+    else return q + (whole(fw) * nu + u0);
+  };
 #pragma unroll 1
   for (int k = 0; k < n_proj; ++k, q += img) {
     const float c = __ldg(cb + k), s = __ldg(sb + k);
@@ -156,9 +166,9 @@ __global__ void __launch_bounds__(256) k_fdk_backproject(const float* __restrict
     const float fu = div_by(u, du_iso, inv_du) + cu;
     // floor(fu) >= 0 and floor(fu) + 1 < nu (false for a NaN)
     const bool u_in = fu >= 0.f && fu < u_top;
-    const float fl = __fadd_rd(fu, kFloor);
-    const int u0 = u_in ? __float_as_int(fl) - 0x4B400000 : 0;
-    const float au = fu - (fl - kFloor);
+    const float fl = floor_of(fu);
+    const int u0 = u_in ? whole(fl) : 0;
+    const float au = fraction(fu, fl);
     const float bu = 1.f - au, m2 = mag * mag;
     if constexpr (ZB <= 2) {
       // few warps: every tap is loaded before any is used (a voxel outside the panel reads a word it leaves out)
@@ -168,10 +178,10 @@ __global__ void __launch_bounds__(256) k_fdk_backproject(const float* __restrict
       for (int j = 0; j < ZB; ++j) {
         const float v = z[j] * mag;
         const float fv = div_by(v, dv_iso, inv_dv) + cv;
-        const float fw = __fadd_rd(fv, kFloor);
-        av[j] = fv - (fw - kFloor);
+        const float fw = floor_of(fv);
+        av[j] = fraction(fv, fw);
         in[j] = u_in && fv >= 0.f && fv < v_top;
-        const float* r0 = q + (in[j] ? (__float_as_int(fw) - 0x4B400000) * nu + u0 : 0);
+        const float* r0 = in[j] ? row(fw, u0) : q;
         t[j][0] = __ldg(r0);
         t[j][1] = __ldg(r0 + 1);
         t[j][2] = __ldg(r0 + nu);
@@ -187,11 +197,11 @@ __global__ void __launch_bounds__(256) k_fdk_backproject(const float* __restrict
       for (int j = 0; j < ZB; ++j) {
         const float v = z[j] * mag;
         const float fv = div_by(v, dv_iso, inv_dv) + cv;
-        const float fw = __fadd_rd(fv, kFloor);
-        const float av = fv - (fw - kFloor);
+        const float fw = floor_of(fv);
+        const float av = fraction(fv, fw);
         float val = 0.f;
         if (u_in && fv >= 0.f && fv < v_top) {
-          const float* r0 = q + ((__float_as_int(fw) - 0x4B400000) * nu + u0);
+          const float* r0 = row(fw, u0);
           const float* r1 = r0 + nu;
           val = (1.f - av) * (bu * __ldg(r0) + au * __ldg(r0 + 1)) + av * (bu * __ldg(r1) + au * __ldg(r1 + 1));
         }
@@ -210,8 +220,9 @@ cudaError_t backproject(const float* q, const float* cb, const float* sb, int n_
                         float scale, float* vol, cudaStream_t s) {
   const long long blocks = (long long)((nx + 15) / 16) * ((ny + 15) / 16) * ((nz + ZB - 1) / ZB);
   if (blocks > 0x7FFFFFFFll) return cudaErrorInvalidValue;
-  k_fdk_backproject<ZB><<<(unsigned)blocks, 256, 0, s>>>(q, cb, sb, n_proj, nu, nv, du, dv, 1.f / du, 1.f / dv, sod, nx, ny,
-                                                         nz, dx, dy, dz, first ? 1 : 0, scale, vol);
+  auto* k = (size_t)nu * nv > 0x7FFFFFFFu || nv > 1 << 22 ? k_fdk_backproject<ZB, true> : k_fdk_backproject<ZB, false>;
+  k<<<(unsigned)blocks, 256, 0, s>>>(q, cb, sb, n_proj, nu, nv, du, dv, 1.f / du, 1.f / dv, sod, nx, ny, nz, dx, dy, dz,
+                                     first ? 1 : 0, scale, vol);
   return cudaGetLastError();
 }
 
