@@ -397,8 +397,8 @@ __global__ void __launch_bounds__(256) k_bin_volume(const uint8_t* __restrict__ 
                                                     uint8_t* __restrict__ mat_b, uint16_t* __restrict__ rho_b) {
   const int bx = nx / 2, by = ny / 2, bz = nz / 2;
   const size_t n = (size_t)bx * by * bz;
-  __shared__ float s_mu[kMaxMat];
-  if (threadIdx.x < kMaxMat) s_mu[threadIdx.x] = murho.v[threadIdx.x];
+  __shared__ float s_mu[256];  // for every id a voxel can hold; one in no table attenuates nothing
+  for (int m = threadIdx.x; m < 256; m += blockDim.x) s_mu[m] = m < n_mat ? murho.v[m] : 0.f;
   __syncthreads();
   // a block's x neighbours as one 2- and one 4-byte word (nx is even, so rows keep the arrays' alignment)
   const bool wide = ((uintptr_t)mat & 1) == 0 && ((uintptr_t)rho & 3) == 0;
