@@ -16,7 +16,7 @@
 // block q of the next level.  So every level reads and writes a thread's own
 // places of one shared array, the frequencies end in digit-reversed places, and
 // the inverse walks the same levels back; multiplying by the kernel's spectrum
-// happens in registers between the two.  368640 rows of 1024: 2.4 ms (1.26 TB/s
+// happens in registers between the two.  368640 rows of 1024: 2.0 ms (1.5 TB/s
 // read and written, bound by issue slots) against 31.9 ms of direct sums.
 #include <stdint.h>
 

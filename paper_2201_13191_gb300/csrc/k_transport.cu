@@ -1317,7 +1317,8 @@ cudaError_t launch_one(const TransportParams& p, int grid, int block, int smem, 
   return cudaGetLastError();
 }
 
-// A packed volume beyond 3/4 of the 126 MB L2 streams from HBM (the line at which the layouts change, too).
+// Words beyond 3/4 of the 126 MB L2 stream from HBM.  (Counted in the layout's own words; the layouts themselves change at
+// 3/4 of the L2 that the device reports, counted in plain words.)
 bool beyond_l2(int layout, int words) { return (double)words * (layout == VOX_HOP2 ? 8.0 : 4.0) > 0.75 * 126e6; }
 
 template <int LAYOUT>

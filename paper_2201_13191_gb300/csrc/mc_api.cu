@@ -118,8 +118,8 @@ MixedLimits mixed_limits(size_t bytes, size_t l2) {
   return {0.25, 0.45};
 }
 
-// Chunk of filtered projections: 256^3 x 360 x 1024^2 takes 13.0 ms with chunks of 128 MB (each launch has its own
-// last wave of blocks), 11.8 with 512 MB.
+// Chunk of filtered projections: 256^3 x 360 x 1024^2 takes 11.4 ms with chunks of 512 MB, and 1.2 ms longer with 128 MB
+// (each launch has its own last wave of blocks).
 constexpr size_t kFdkChunk = (size_t)512 << 20;
 
 int fail(mc_ctx* c, int code, const std::string& msg) {
