@@ -346,8 +346,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv3x3_fwd(const __grid_consta
 // leaves out the columns of the dy that falls outside, so that a value that is
 // not finite meets the same products as in the sum above.  Where the width is no
 // multiple of 16 such a value also meets the zeros beside the image (in the last
-// column's dx = -1; in 8-wide tiles in the first or last row's third dy): there
-// the accumulators that are not finite are summed again from global memory.
+// column's dx = -1; in 8-wide tiles in the first or last row's third dy): the
+// accumulators that this has spoilt are summed again from global memory.
 //
 // CTA (cin chunk, cout tile, split): the split's tiles, a run of neighbours (its
 // partial sums then grow, and round, like those of a run of pixels), go through a
@@ -384,26 +384,49 @@ struct WgArgs {
   int* err;
 };
 
-// dW[co][tap_y, tap_x][c] over `count` tiles from `first` on, the products inside the image only.
-__device__ __noinline__ float wgrad_direct(WgArgs p, long long first, int count, int c, int co, int tap_y, int tap_x) {
+// dW[co .. co + 7][tap_y, tap_x][c] over `count` tiles from `first` on, the products inside the image only.
+__device__ __forceinline__ void wgrad_direct(const WgArgs& p, long long first, int count, int c, int co, int tap_y,
+                                             int tap_x, float (&sum)[8]) {
   const int per_img = p.tiles_x * p.tiles_y;
-  float sum = 0.f;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) sum[i] = 0.f;
   for (long long t = first; t < first + count; ++t) {
     const long long img = t / per_img;
     const int r = (int)(t - img * per_img), y0 = (r / p.tiles_x) * p.ty, x0 = (r % p.tiles_x) * p.tx;
-    for (int y = y0; y < min(y0 + p.ty, p.h); ++y) {
-      const int gy = y - (tap_y - 1);
-      if (gy < 0 || gy >= p.h) continue;
-      const __nv_bfloat16* row_x = p.x + (img * p.h + y) * p.w * p.cin + c;
-      const __nv_bfloat16* row_g = p.dy + (img * p.h + gy) * p.w * p.cout + co;
-      for (int x = x0; x < min(x0 + p.tx, p.w); ++x) {
-        const int px = x + tap_x - 1;
-        if (px >= 0 && px < p.w)
-          sum = fmaf(__bfloat162float(row_x[(long long)px * p.cin]), __bfloat162float(row_g[(long long)x * p.cout]), sum);
+    const int xa = max(x0, 1 - tap_x), xb = min(min(x0 + p.tx, p.w), p.w + 1 - tap_x);
+    for (int y = max(y0, tap_y - 1); y < min(min(y0 + p.ty, p.h), p.h + tap_y - 1); ++y) {
+      const __nv_bfloat16* row_x = p.x + ((img * p.h + y) * p.w + (tap_x - 1)) * p.cin + c;
+      const __nv_bfloat16* row_g = p.dy + (img * p.h + y - (tap_y - 1)) * p.w * p.cout + co;
+#pragma unroll 4
+      for (int x = xa; x < xb; ++x) {
+        const float v = __bfloat162float(row_x[(long long)x * p.cin]);
+        const uint4 q = __ldg(reinterpret_cast<const uint4*>(row_g + (long long)x * p.cout));
+        const uint32_t g[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          sum[i] = fmaf(v, __uint_as_float(i & 1 ? g[i >> 1] & 0xFFFF0000u : g[i >> 1] << 16), sum[i]);
       }
+      bool nan = true;  // all of them: they stay no numbers
+#pragma unroll
+      for (int i = 0; i < 8; ++i) nan &= sum[i] != sum[i];
+      if (nan) return;
     }
   }
-  return sum;
+}
+
+// Whether channel c holds a value that is not finite in the last column of `count` tiles from `first` on.
+__device__ __forceinline__ bool wgrad_last_column(const WgArgs& p, long long first, int count, int c) {
+  const int per_img = p.tiles_x * p.tiles_y;
+  float z = 0.f;
+  for (long long t = first; t < first + count; ++t) {
+    const long long img = t / per_img;
+    const int r = (int)(t - img * per_img), y0 = (r / p.tiles_x) * p.ty;
+    if (r % p.tiles_x != p.tiles_x - 1) continue;
+#pragma unroll 4
+    for (int y = y0; y < min(y0 + p.ty, p.h); ++y)
+      z = fmaf(__bfloat162float(p.x[((img * p.h + y) * p.w + p.w - 1) * p.cin + c]), 0.f, z);
+  }
+  return z != 0.f;
 }
 
 // RAGGED: the width is no multiple of 16 (a variant of its own: the sums from global memory double the registers).
@@ -524,6 +547,9 @@ __global__ void __launch_bounds__(kThreads) k_conv3x3_wgrad(const __grid_constan
       again = __any_sync(0xFFFFFFFFu, again);
     }
     if (RAGGED && again) {
+      // zeros beside the image have met the last column's values in the dx = -1 taps, and in 8-wide tiles values of the
+      // first and last row in a third dy
+      const bool edge = p.tx == 8 || wgrad_last_column(p, first, count, c0 + c);
 #pragma unroll 1
       for (int j = 0; j < P::cols; j += 8) {
         float v[8];
@@ -531,14 +557,17 @@ __global__ void __launch_bounds__(kThreads) k_conv3x3_wgrad(const __grid_constan
         tc::tmem_ld8(lane_base + (uint32_t)j, v);
         const int a = j / NT, n = n0 + j % NT;
         if (blk + 2 * (a / 3) >= 3) continue;
-#pragma unroll 1
-        for (int i = 0; i < 8; ++i) {
-          float o = v[0];
+        bool finite = true;
 #pragma unroll
-          for (int q = 1; q < 8; ++q) o = q == i ? v[q] : o;
-          if (!(fabsf(o) < INFINITY)) o = wgrad_direct(p, first, count, c0 + c, n + i, tap(a) / 3, tap(a) % 3);
-          atomicAdd(p.dw + ((size_t)(n + i) * 9 + tap(a)) * p.cin + c0 + c, o);
+        for (int i = 0; i < 8; ++i) finite &= fabsf(v[i]) < INFINITY;
+        if (!finite && edge && (p.tx == 8 || tap(a) % 3 == 0)) {
+          float o[8];
+          wgrad_direct(p, first, count, c0 + c, n, tap(a) / 3, tap(a) % 3, o);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) v[i] = fabsf(v[i]) < INFINITY ? v[i] : o[i];
         }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) atomicAdd(p.dw + ((size_t)(n + i) * 9 + tap(a)) * p.cin + c0 + c, v[i]);
       }
     } else {
 #pragma unroll 1
